@@ -109,13 +109,13 @@ struct __align__(128) CorrSmem {
 };
 
 // Swizzle of a plane (rows of kTC = 128 bytes, 8 chunks of 16): chunk c of
-// row e sits at chunk c ^ f(e), f(e) = (e ^ (e >> 3)) & 7. Eight consecutive
-// rows then hit eight different 16-byte bank groups (ldmatrix, the dp4a
-// operand loads), and so do the unpack stores below (rows 4eg + slot across a
-// quarter-warp).
+// row e sits at chunk c ^ (e & 7). Eight consecutive rows then hit eight
+// different 16-byte bank groups (ldmatrix, the dp4a operand loads), rows 8
+// apart share their swizzle (so a lane's rows are immediate offsets from one
+// address), and the unpack stores below (rows 4eg + slot across a
+// quarter-warp) are free of conflicts through their slot order.
 __device__ __forceinline__ uint32_t plane_off(int e, int chunk) {
-  const int f = (e ^ (e >> 3)) & 7;
-  return static_cast<uint32_t>(e * kTC + ((chunk ^ f) << 4));
+  return static_cast<uint32_t>(e * kTC + ((chunk ^ (e & 7)) << 4));
 }
 
 // ---- unpack: packed box [time][element] -> planes [element][time] --------------
@@ -127,33 +127,44 @@ __device__ __forceinline__ uint32_t plane_off(int e, int chunk) {
 //   v - 8      = (v + 0x78) ^ 0x80
 //   hi + lo - 16 = (hi + lo + 0x70) ^ 0x80      (xr + xi)
 //   hi - lo    = ((hi | 0x80) - lo) ^ 0x80       (xr - xi)
-// Lanes 16..31 load their rows in the order k ^ 1 and odd element quads
-// store their elements in the order slot ^ 1, so that loads and stores are
-// free of bank conflicts; runtime prmt selectors undo both reorderings.
+// Rows are loaded in the order k ^ rx, with bit 0 of rx set for lanes 16..31,
+// and element quad eg stores its elements in the order slot ^ (eg >> 1 & 3),
+// so that loads and stores are free of bank conflicts; runtime prmt selectors
+// undo both reorderings. Bit 2 of rx (a multiple of four rows, so the
+// selectors do not see it) leaves the two words of every 8 samples swapped in
+// the planes.
 //
 // kEnc (offset-encoded operands, the Eq. 3 route): the planes keep the
 // encoded nibbles, all unsigned: Xr = hi, Xi = lo, Xr + Xi = hi + lo (row
 // side) and Xr - Xi + 15 = (hi + 15) - lo (column side), each in [0, 30];
 // masked rows are 0x00, which zeroes every product they enter (each product
 // has a row-side factor Xr, Xi or Xr + Xi).
+//
+// pl0, pl1, pls, pld: the planes xr, xi, xr + xi and xr - xi (0 = not wanted).
 template <bool kMasked, bool kEnc>
-__device__ __forceinline__ void unpack_unit(const uint8_t* box, uint32_t pl0, uint32_t pl1, uint32_t pl2,
-                                            bool side_b, int eg, int tg, int p, int lo, int hi, int lo2 = 0,
-                                            int hi2 = 0) {
+__device__ __forceinline__ void unpack_load(const uint8_t* box, int eg, int tg, int rx, int lo, int hi, int lo2,
+                                            int hi2, uint32_t (&r)[16]) {
   const uint32_t* w = reinterpret_cast<const uint32_t*>(box);
-  uint32_t r[16];
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
-    const int t = 16 * tg + (k ^ p);
+    const int t = 16 * tg + (k ^ rx);
     r[k] = w[t * (kTile / 4) + eg];
     // rows outside [lo, hi) and [lo2, hi2): no products
     if (kMasked) r[k] = ((t >= lo && t < hi) || (t >= lo2 && t < hi2)) ? r[k] : (kEnc ? 0u : 0x88888888u);
   }
-  const int s = eg & 1;
-  const uint32_t selA = p ? 0x1504u : 0x5140u;  // interleave two rows, bytes 0-1
-  const uint32_t selB = p ? 0x3726u : 0x7362u;  // bytes 2-3
-  const uint32_t lo16 = s ? 0x7632u : 0x5410u;  // slots 0 / 2: element (slot ^ s)
-  const uint32_t hi16 = s ? 0x5410u : 0x7632u;  // slots 1 / 3
+}
+
+template <bool kEnc>
+__device__ __forceinline__ void unpack_store(const uint32_t (&r)[16], uint32_t pl0, uint32_t pl1, uint32_t pls,
+                                             uint32_t pld, int eg, int tg, int rx) {
+  const int p = rx & 1;
+  const int s = (eg >> 1) & 3;
+  const uint32_t sel01 = p ? 0x1504u : 0x5140u;  // interleave two rows, bytes 0-1
+  const uint32_t sel23 = p ? 0x3726u : 0x7362u;  // bytes 2-3
+  const uint32_t selA = s & 2 ? sel23 : sel01;   // slots 0-1: elements (slot ^ s)
+  const uint32_t selB = s & 2 ? sel01 : sel23;   // slots 2-3
+  const uint32_t lo16 = s & 1 ? 0x7632u : 0x5410u;  // slots 0 / 2
+  const uint32_t hi16 = s & 1 ? 0x5410u : 0x7632u;  // slots 1 / 3
   uint32_t wd[4][4];  // [slot][time quad]
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
@@ -169,26 +180,43 @@ __device__ __forceinline__ void unpack_unit(const uint8_t* box, uint32_t pl0, ui
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const int e = 4 * eg + (k ^ s);
-    uint32_t xr[4], xi[4], sd[4];
+    const uint32_t off = plane_off(e, tg);
+    uint32_t hi[4], lo[4], v[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const uint32_t hi = (wd[k][j] >> 4) & 0x0F0F0F0Fu;
-      const uint32_t lo = wd[k][j] & 0x0F0F0F0Fu;
-      if (kEnc) {
-        xr[j] = hi;
-        xi[j] = lo;
-        sd[j] = side_b ? ((hi + 0x0F0F0F0Fu) - lo) : (hi + lo);
-      } else {
-        xr[j] = (hi + 0x78787878u) ^ 0x80808080u;
-        xi[j] = (lo + 0x78787878u) ^ 0x80808080u;
-        sd[j] = side_b ? (((hi | 0x80808080u) - lo) ^ 0x80808080u) : ((hi + lo + 0x70707070u) ^ 0x80808080u);
-      }
+      hi[j] = (wd[k][j] >> 4) & 0x0F0F0F0Fu;
+      lo[j] = wd[k][j] & 0x0F0F0F0Fu;
     }
-    const uint32_t off = plane_off(e, tg);
-    if (pl0) sts128(pl0 + off, xr[0], xr[1], xr[2], xr[3]);  // (0 = plane not wanted)
-    if (pl1) sts128(pl1 + off, xi[0], xi[1], xi[2], xi[3]);
-    sts128(pl2 + off, sd[0], sd[1], sd[2], sd[3]);
+    if (pls) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[j] = kEnc ? hi[j] + lo[j] : (hi[j] + lo[j] + 0x70707070u) ^ 0x80808080u;
+      sts128(pls + off, v[0], v[1], v[2], v[3]);
+    }
+    if (pld) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        v[j] = kEnc ? (hi[j] + 0x0F0F0F0Fu) - lo[j] : ((hi[j] | 0x80808080u) - lo[j]) ^ 0x80808080u;
+      sts128(pld + off, v[0], v[1], v[2], v[3]);
+    }
+    if (pl0) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (!kEnc) hi[j] = (hi[j] + 0x78787878u) ^ 0x80808080u;
+        if (!kEnc) lo[j] = (lo[j] + 0x78787878u) ^ 0x80808080u;
+      }
+      sts128(pl0 + off, hi[0], hi[1], hi[2], hi[3]);
+      sts128(pl1 + off, lo[0], lo[1], lo[2], lo[3]);
+    }
   }
+}
+
+template <bool kMasked, bool kEnc>
+__device__ __forceinline__ void unpack_unit(const uint8_t* box, uint32_t pl0, uint32_t pl1, uint32_t pl2,
+                                            bool side_b, int eg, int tg, int rx, int lo, int hi, int lo2 = 0,
+                                            int hi2 = 0) {
+  uint32_t r[16];
+  unpack_load<kMasked, kEnc>(box, eg, tg, rx, lo, hi, lo2, hi2, r);
+  unpack_store<kEnc>(r, pl0, pl1, side_b ? 0u : pl2, side_b ? pl2 : 0u, eg, tg, rx);
 }
 
 // ---- product: one 128-sample chunk of a warp's 16 x 16 piece of the tile --------
@@ -414,7 +442,7 @@ __device__ __forceinline__ void gate_windows(int32_t c, int32_t T, int32_t P, in
 // (the current one c, the next one cn).
 template <bool kFrames, bool kHold, bool kArith = false>
 struct Walk {
-  int item, c, f, bi, bj, c1, frame, T, nch, T0;
+  int item, c, c0, f, bi, bj, c1, frame, T, nch, T0;
   const int4* items;
   const FrameDesc* frames;
   int nitems, stride;
@@ -429,7 +457,7 @@ struct Walk {
     for (; item < nitems; item += stride) {
       const int4 w = items[item];
       bi = w.y & 0xFFFF;
-      c = w.z;
+      c = c0 = w.z;
       c1 = w.w;
       if (kFrames) {
         bj = kHold ? (w.y >> 16) & 0x7FFF : w.y >> 16;  // (bit 31: hold, read by the writer)
@@ -481,6 +509,20 @@ struct Walk {
     T0 = 0;
     load();
   }
+  // As start(), one step before the first unit: next() goes there.
+  __device__ __forceinline__ void before(const CorrArgs& a) {
+    items = a.items;
+    frames = a.frames;
+    nitems = a.nitems;
+    stride = gridDim.x;
+    item = static_cast<int>(blockIdx.x) - stride;
+    frame = -1;
+    T = a.T;
+    nch = a.nch;
+    T0 = 0;
+    c = -1;
+    c1 = cn = 0;
+  }
   __device__ __forceinline__ bool valid() const { return item < nitems; }
   // the current chunk is the item's last
   __device__ __forceinline__ bool last() const { return kArith ? cn >= c1 : c + 1 == c1; }
@@ -514,14 +556,14 @@ constexpr uint32_t kDiagR = 0xfa9050u, kDiagC = 0xfaedd8u, kDiagSel = 0xff990000
 // Split of a chunk's 128 samples between the tensor cores (k-steps of 32)
 // and dp4a (the rest), chosen per launch: the same split for every chunk, or
 // two splits alternating between consecutive chunks of a CTA, which gives the
-// finer average shares in between. Shares 5 and 4 apply to off-diagonal
+// finer average shares in between. Share 4 applies to off-diagonal
 // tiles; diagonal tiles keep 6. Every split gives the same exact sums.
 // Tensor-core k-steps per pair of chunks:
 enum : int {
   kSplitMma = 0,   // 8 of 8: tensor cores only
   kSplit6 = 1,     // 6 of 8 (96 / 32 per chunk)
   kSplit7 = 2,     // 7 of 8 (alternating 128 / 0 and 96 / 32)
-  kSplit5 = 3,     // 5 of 8 (alternating 64 / 64 and 96 / 32)
+  kSplitDual = 3,  // not this kernel: the dual-engine kernel of xe_dual.cuh
   kSplit4 = 4      // 4 of 8 (64 / 64 per chunk)
 };
 
@@ -530,7 +572,6 @@ __device__ __forceinline__ int mma_ksteps(int hybrid, int odd) {
   switch (hybrid) {
     case kSplit6: return 3;
     case kSplit7: return odd ? 4 : 3;
-    case kSplit5: return odd ? 2 : 3;
     case kSplit4: return 2;
     default: return 4;
   }
@@ -565,10 +606,10 @@ __device__ __forceinline__ void product_chunk(CorrSmem& sm, int buf, int warp, i
   const uint32_t b_side = smem_u32(sm.plane[buf][1][0]);
   const uint32_t b01 = diag ? a_base : b_side, b2 = b_side + kPsd * kPlaneBytes;
   const int ksteps = nvalid >= kTC ? kTC / 32 : (nvalid + 31) / 32;
-  // shares below 6 apply to off-diagonal tiles: a diagonal tile, with a quarter of its product warps
+  // share 4 applies to off-diagonal tiles: a diagonal tile, with a quarter of its product warps
   // idle and a quarter on single sub-tiles, runs best at 6 (measured)
   const int split0 = kSplitT < 0 ? (hybrid == kSplitMma ? kSplitMma : kSplit6) : kSplitT;
-  const int split = diag && (split0 == kSplit5 || split0 == kSplit4) ? kSplit6 : split0;
+  const int split = diag && split0 == kSplit4 ? kSplit6 : split0;
   if (split != kSplitMma && ksteps == kTC / 32) {  // (a ragged last chunk takes the tensor-core path)
     const int mk = mma_ksteps(split, static_cast<int>(it & 1));
     if (sel == kSelAll)

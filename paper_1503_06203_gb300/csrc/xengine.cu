@@ -15,6 +15,7 @@
 #include "xengine.h"
 #include "xe_batch.cuh"
 #include "xe_corr.cuh"
+#include "xe_dual.cuh"
 #include "xe_lags.cuh"
 #include "xe_offsets.cuh"
 
@@ -53,6 +54,8 @@ EncodeTiledFn encode_fn() {
 
 // ---- per-device kernel set-up ---------------------------------------------------
 constexpr size_t kSmemBytes = sizeof(xe::CorrSmem) + 128;  // + alignment slack
+constexpr size_t kDualSmemBytes = sizeof(xe::DualSmem) + 128;
+static_assert(kSmemBytes <= 232448 && kDualSmemBytes <= 232448, "shared memory of one CTA");
 std::mutex g_dev_mu;
 int g_blocks_per_sm[64];
 int g_sms[64];
@@ -65,7 +68,6 @@ int device_setup(int dev) {
   cudaError_t e = cudaSuccess;
   for (const void* k : {reinterpret_cast<const void*>(xe::corr_tile_kernel<xe::kSingle, false>),
                         reinterpret_cast<const void*>(xe::corr_tile_kernel<xe::kSingle, false, xe::kSplit7>),
-                        reinterpret_cast<const void*>(xe::corr_tile_kernel<xe::kSingle, false, xe::kSplit5>),
                         reinterpret_cast<const void*>(xe::corr_tile_kernel<xe::kSingle, false, xe::kSplit4>),
                         reinterpret_cast<const void*>(xe::corr_tile_kernel<xe::kBatch, false>),
                         reinterpret_cast<const void*>(xe::corr_tile_kernel<xe::kGated, false>),
@@ -73,7 +75,17 @@ int device_setup(int dev) {
                         reinterpret_cast<const void*>(xe::corr_tile_kernel<xe::kSingle, true>)})
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemBytes));
-  if (e != cudaSuccess) return fail(CORR_ECUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
+  for (const void* k : {reinterpret_cast<const void*>(xe::corr_dual_kernel<xe::kSingle>),
+                        reinterpret_cast<const void*>(xe::corr_dual_kernel<xe::kBatch>)}) {
+    // its register re-split draws on the registers it is launched with: fewer would leave it waiting for good
+    cudaFuncAttributes at;
+    e = cudaFuncGetAttributes(&at, k);
+    if (e == cudaSuccess && at.numRegs < xe::kRegsLaunch)
+      return fail(CORR_ECUDA, "the correlator was built with %d registers a thread, not %d", at.numRegs, xe::kRegsLaunch);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kDualSmemBytes));
+    if (e != cudaSuccess) return fail(CORR_ECUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
+  }
   int bps = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, xe::corr_tile_kernel<xe::kSingle, false>, xe::kThreads,
                                                     kSmemBytes);
@@ -115,7 +127,7 @@ int chunk_hybrid_flag(int product, int mma_steps) {
   switch (mma_steps) {
     case 8: return xe::kSplitMma;
     case 7: return xe::kSplit7;
-    case 5: return xe::kSplit5;
+    case 5: return xe::kSplitDual;
     case 4: return xe::kSplit4;
     default: return xe::kSplit6;
   }
@@ -424,8 +436,8 @@ int launch_frame(corr_handle* h, const uint8_t* frame, int32_t Np, int64_t row_b
     xe::corr_tile_kernel<xe::kSingle, true><<<pl.grid, xe::kThreads, kSmemBytes, st>>>(tm, a);
   else if (a.hybrid == xe::kSplit7)
     xe::corr_tile_kernel<xe::kSingle, false, xe::kSplit7><<<pl.grid, xe::kThreads, kSmemBytes, st>>>(tm, a);
-  else if (a.hybrid == xe::kSplit5)
-    xe::corr_tile_kernel<xe::kSingle, false, xe::kSplit5><<<pl.grid, xe::kThreads, kSmemBytes, st>>>(tm, a);
+  else if (a.hybrid == xe::kSplitDual)
+    xe::corr_dual_kernel<xe::kSingle><<<pl.grid, xe::kDualThreads, kDualSmemBytes, st>>>(tm, a);
   else if (a.hybrid == xe::kSplit4)
     xe::corr_tile_kernel<xe::kSingle, false, xe::kSplit4><<<pl.grid, xe::kThreads, kSmemBytes, st>>>(tm, a);
   else
@@ -609,6 +621,28 @@ int grow_set(BatchSet& b, size_t frames, size_t items) {
   return CORR_OK;
 }
 
+// The correlator of a batched launch: the default share runs the dual-engine
+// kernel, every other one the runtime-split kernel (as 8 or 6). Gated launches
+// run the runtime-split kernel.
+struct CorrLaunch {
+  void* fn;
+  unsigned threads, smem;
+};
+
+CorrLaunch corr_launch_of(int mode, int hybrid) {
+  if (hybrid == xe::kSplitDual)
+    return {reinterpret_cast<void*>(xe::corr_dual_kernel<xe::kBatch>), xe::kDualThreads, static_cast<unsigned>(kDualSmemBytes)};
+  return {mode == xe::kBatch   ? reinterpret_cast<void*>(xe::corr_tile_kernel<xe::kBatch, false>)
+          : mode == xe::kGated ? reinterpret_cast<void*>(xe::corr_tile_kernel<xe::kGated, false>)
+                               : reinterpret_cast<void*>(xe::corr_tile_kernel<xe::kGateArith, false>),
+          xe::kThreads, static_cast<unsigned>(kSmemBytes)};
+}
+
+// The split a batched or gated launch runs: the runtime-split kernel knows tensor cores only and 6 of 8.
+int shared_split(int hybrid, bool gated) {
+  return hybrid == xe::kSplitMma || (hybrid == xe::kSplitDual && !gated) ? hybrid : xe::kSplit6;
+}
+
 // kind: 1 = gate segments (corr_tile_kernel<kGated>), 2 = gate arithmetic (<kGateArith>).
 int build_graph(BatchSet& b, int64_t nframes, int64_t nitems, int64_t grid, int32_t* err, int hybrid, int kind) {
   if (b.exec) {
@@ -641,11 +675,11 @@ int build_graph(BatchSet& b, int64_t nframes, int64_t nitems, int64_t grid, int3
   void* params[2] = {&unused, &a};
   cudaKernelNodeParams kp;
   memset(&kp, 0, sizeof kp);
-  kp.func = kind == 1 ? reinterpret_cast<void*>(xe::corr_tile_kernel<xe::kGated, false>)
-                      : reinterpret_cast<void*>(xe::corr_tile_kernel<xe::kGateArith, false>);
+  const CorrLaunch cl = corr_launch_of(kind == 1 ? xe::kGated : xe::kGateArith, hybrid);
+  kp.func = cl.fn;
   kp.gridDim = dim3(static_cast<unsigned>(grid));
-  kp.blockDim = dim3(xe::kThreads);
-  kp.sharedMemBytes = static_cast<unsigned>(kSmemBytes);
+  kp.blockDim = dim3(cl.threads);
+  kp.sharedMemBytes = cl.smem;
   kp.kernelParams = params;
   if (e == cudaSuccess) e = cudaGraphAddKernelNode(&kn, g, cp, 2, &kp);
   if (e == cudaSuccess) e = cudaGraphInstantiate(&b.exec, g, 0);
@@ -744,13 +778,6 @@ int ring_set_items(RingSet& r, int64_t nitems, cudaStream_t st) {
   return CORR_OK;
 }
 
-// Batched launches run kSplitMma or kSplit6, chosen at run time (other shares run as 6: a share-5
-// instantiation of the batch kernel spilled and measured slower than share 6).
-void* corr_kernel_fn(int hybrid) {
-  (void)hybrid;
-  return reinterpret_cast<void*>(xe::corr_tile_kernel<xe::kBatch, false>);
-}
-
 // Set the three nodes' parameters from r.p_* (and build the graph the first time).
 int ring_set_launch(RingSet& r, int hybrid, cudaStream_t st) {
   const unsigned plan_blocks = static_cast<unsigned>(std::min<int64_t>(ceil_div(r.p_nitems, 256), 4096));
@@ -763,10 +790,11 @@ int ring_set_launch(RingSet& r, int hybrid, cudaStream_t st) {
   kp_plan.blockDim = dim3(256);
   kp_plan.kernelParams = plan_params;
   memset(&kp_corr, 0, sizeof kp_corr);
-  kp_corr.func = corr_kernel_fn(hybrid);
+  const CorrLaunch cl = corr_launch_of(xe::kBatch, hybrid);
+  kp_corr.func = cl.fn;
   kp_corr.gridDim = dim3(static_cast<unsigned>(r.p_grid));
-  kp_corr.blockDim = dim3(xe::kThreads);
-  kp_corr.sharedMemBytes = static_cast<unsigned>(kSmemBytes);
+  kp_corr.blockDim = dim3(cl.threads);
+  kp_corr.sharedMemBytes = cl.smem;
   kp_corr.kernelParams = corr_params;
   cudaError_t e = cudaSuccess;
   if (r.exec) {  // update the instantiated graph in place; rebuild it if the update is refused
@@ -989,7 +1017,7 @@ static int batch_shared(corr_handle_t* const* hs, const uint8_t* const* inputs, 
     d.nb = static_cast<int32_t>(ceil_div(h->N, xe::kTile));
     d.per = static_cast<int32_t>(per[k]);
   }
-  const int hybrid = chunk_hybrid_flag(hs[0]->product, hs[0]->mma_steps);
+  const int hybrid = shared_split(chunk_hybrid_flag(hs[0]->product, hs[0]->mma_steps), false);
   r.p_frames = reinterpret_cast<const xe::FrameDesc*>(r.d_blk);
   r.p_first = reinterpret_cast<const int64_t*>(r.d_blk + kFirstOff);
   r.p_order = reinterpret_cast<const int32_t*>(r.d_blk + kOrderOff);
@@ -1007,7 +1035,7 @@ static int batch_shared(corr_handle_t* const* hs, const uint8_t* const* inputs, 
   a.B = 0;
   a.vis = nullptr;
   a.fresh = 0;
-  a.hybrid = hybrid == xe::kSplitMma ? xe::kSplitMma : xe::kSplit6;  // (the runtime-split instantiation's choice)
+  a.hybrid = hybrid;
   a.err = hs[0]->d_err;
   if ((rc = ring_set_launch(r, hybrid, st))) return rc;
   ring.next = (ring.next + 1) % kBatchSets;
@@ -1084,7 +1112,7 @@ int gated_arith_launch(corr_handle_t* const* gates, int G, const CUtensorMap& ma
     d.G = G;
     d.gate = g;
   }
-  const int hybrid = chunk_hybrid_flag(h0->product, h0->mma_steps) == xe::kSplitMma ? xe::kSplitMma : xe::kSplit6;
+  const int hybrid = shared_split(chunk_hybrid_flag(h0->product, h0->mma_steps), true);
   if (!b.exec || b.key_frames != G || b.key_items != nitems || b.key_grid != grid || b.key_hybrid != hybrid ||
       b.key_gated != 2 || b.key_err != h0->d_err)
     if ((rc = build_graph(b, G, nitems, grid, h0->d_err, hybrid, 2))) return rc;
@@ -1246,7 +1274,7 @@ int gated_impl(corr_handle_t* const* gates, int G, const uint8_t* in, int32_t T,
     d.t0 = empty ? 1 : segs[s].t0;  // t0 > T: nothing is valid
     d.atomic = 0;
   }
-  const int hybrid = chunk_hybrid_flag(h0->product, h0->mma_steps) == xe::kSplitMma ? xe::kSplitMma : xe::kSplit6;
+  const int hybrid = shared_split(chunk_hybrid_flag(h0->product, h0->mma_steps), true);
   if (!b.exec || b.key_frames != nseg || b.key_items != nitems || b.key_grid != grid || b.key_hybrid != hybrid ||
       b.key_gated != 1 || b.key_err != h0->d_err)
     if ((rc = build_graph(b, nseg, nitems, grid, h0->d_err, hybrid, 1))) return rc;
@@ -1853,10 +1881,10 @@ extern "C" int corr_correlate_noalloc(const uint8_t* packed_dev, int32_t N, int3
   a.B = static_cast<int64_t>(N) * (N + 1) / 2;
   a.vis = vis_dev;
   a.fresh = 1;
-  a.hybrid = 0;
+  a.hybrid = xe::kSplitDual;
   a.err = reinterpret_cast<int32_t*>(scratch);
   const int grid = static_cast<int>(std::min<int64_t>(slots, nitems));
-  xe::corr_tile_kernel<xe::kSingle, false><<<grid, xe::kThreads, kSmemBytes, st>>>(tm, a);
+  xe::corr_dual_kernel<xe::kSingle><<<grid, xe::kDualThreads, kDualSmemBytes, st>>>(tm, a);
   if ((e = cudaGetLastError()) != cudaSuccess) return fail(CORR_ECUDA, "noalloc correlate: %s", cudaGetErrorString(e));
   if (status_dev && (e = cudaMemcpyAsync(status_dev, scratch, sizeof(int32_t), cudaMemcpyDeviceToDevice, st)) !=
                         cudaSuccess)
