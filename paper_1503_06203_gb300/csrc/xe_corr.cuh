@@ -88,8 +88,7 @@ struct CorrArgs {
 struct ChunkMeta {
   int32_t f;        // band
   int32_t bij;      // bi | bj << 16
-  int32_t lo, hi;   // valid rows of the chunk: [lo, hi) and [lo2, hi2)
-  int32_t lo2, hi2;
+  int32_t lo, hi;   // valid rows of the chunk: [lo, hi)
   int32_t flags;    // kMetaValid | kMetaEnd | write mode << 4 (kMetaEnd unset while a gated group holds)
   int32_t N;
   int64_t B;
@@ -142,15 +141,15 @@ __device__ __forceinline__ uint32_t plane_off(int e, int chunk) {
 //
 // pl0, pl1, pls, pld: the planes xr, xi, xr + xi and xr - xi (0 = not wanted).
 template <bool kMasked, bool kEnc>
-__device__ __forceinline__ void unpack_load(const uint8_t* box, int eg, int tg, int rx, int lo, int hi, int lo2,
-                                            int hi2, uint32_t (&r)[16]) {
+__device__ __forceinline__ void unpack_load(const uint8_t* box, int eg, int tg, int rx, int lo, int hi,
+                                            uint32_t (&r)[16]) {
   const uint32_t* w = reinterpret_cast<const uint32_t*>(box);
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
     const int t = 16 * tg + (k ^ rx);
     r[k] = w[t * (kTile / 4) + eg];
-    // rows outside [lo, hi) and [lo2, hi2): no products
-    if (kMasked) r[k] = ((t >= lo && t < hi) || (t >= lo2 && t < hi2)) ? r[k] : (kEnc ? 0u : 0x88888888u);
+    // rows outside [lo, hi): no products
+    if (kMasked) r[k] = (t >= lo && t < hi) ? r[k] : (kEnc ? 0u : 0x88888888u);
   }
 }
 
@@ -212,10 +211,9 @@ __device__ __forceinline__ void unpack_store(const uint32_t (&r)[16], uint32_t p
 
 template <bool kMasked, bool kEnc>
 __device__ __forceinline__ void unpack_unit(const uint8_t* box, uint32_t pl0, uint32_t pl1, uint32_t pl2,
-                                            bool side_b, int eg, int tg, int rx, int lo, int hi, int lo2 = 0,
-                                            int hi2 = 0) {
+                                            bool side_b, int eg, int tg, int rx, int lo, int hi) {
   uint32_t r[16];
-  unpack_load<kMasked, kEnc>(box, eg, tg, rx, lo, hi, lo2, hi2, r);
+  unpack_load<kMasked, kEnc>(box, eg, tg, rx, lo, hi, r);
   unpack_store<kEnc>(r, pl0, pl1, side_b ? 0u : pl2, side_b ? pl2 : 0u, eg, tg, rx);
 }
 
@@ -397,49 +395,19 @@ __device__ __forceinline__ void write_piece(int N, int64_t B, int32_t* vis, int 
 // unpack; lane 0 of warp 16 also issues the TMA loads. One CTA per SM.
 
 // ---- gate arithmetic (kGateArith launches) --------------------------------------
-// Gate g of G holds the positions [a, b) of a period P, a = ceil(g P / G),
-// b = ceil((g + 1) P / G): floor(pos G / P) == g exactly there. Sample t has
-// position (t + phase) mod P. Chunks are kTC samples; P >= kTC, so a chunk's
-// positions wrap at most once and the gate meets a chunk in at most two runs.
-// 32-bit unsigned arithmetic is exact: sample indices are below 2^31 and the
-// host takes this route only for P <= 2^29, so sample + phase and
-// sample + 2P stay below 2^32.
-
-// The first sample >= s whose position lies in [a, b) (a < b <= P).
-__device__ __forceinline__ uint32_t gate_next_sample(uint32_t s, uint32_t P, uint32_t phase, uint32_t a, uint32_t b) {
-  const uint32_t pos = (s + phase) % P;
-  if (pos >= a && pos < b) return s;
-  return s + (pos < a ? a - pos : P - pos + a);
-}
-
-// The first chunk >= c holding a sample t < T of the gate; nch if none.
-__device__ __forceinline__ int32_t gate_chunk(int32_t c, int32_t nch, int32_t T, int32_t P, int32_t phase, int32_t a,
-                                              int32_t b) {
-  if (c >= nch || a >= b) return nch;
-  const uint32_t s = gate_next_sample(static_cast<uint32_t>(c) * kTC, static_cast<uint32_t>(P),
-                                      static_cast<uint32_t>(phase), static_cast<uint32_t>(a), static_cast<uint32_t>(b));
-  return s >= static_cast<uint32_t>(T) ? nch : static_cast<int32_t>(s / kTC);
-}
-
-// The gate's rows of chunk c (relative to its first sample), as two windows
-// [lo, hi) and [lo2, hi2): the run before the chunk's positions wrap past P
-// and the run after it; both clipped to the frame's T samples.
-__device__ __forceinline__ void gate_windows(int32_t c, int32_t T, int32_t P, int32_t phase, int32_t a, int32_t b,
-                                             ChunkMeta& m) {
-  const uint32_t s0 = static_cast<uint32_t>(c) * kTC;
-  const int32_t p0 = static_cast<int32_t>((s0 + static_cast<uint32_t>(phase)) % static_cast<uint32_t>(P));
-  const int32_t tmax = min(kTC, T - static_cast<int32_t>(s0));
-  m.lo = max(0, a - p0);
-  m.hi = min(tmax, b - p0);
-  m.lo2 = max(0, a - p0 + P);
-  m.hi2 = min(tmax, b - p0 + P);
-}
+// Gate g of G holds the positions [ga, gb) of a period P, ga = ceil(g P / G),
+// gb = ceil((g + 1) P / G): floor(pos G / P) == g exactly there. Sample t has
+// position (t + phase) mod P. The gate's samples are runs of gb - ga, P apart
+// (the frame's ends may cut the first and the last). An item's chunks start
+// at the runs' first samples, not at multiples of kTC (TMA takes any time
+// coordinate), so a run of up to kTC samples is one chunk: with 8 gates of
+// 1024 samples and a phase of 100, half the chunks that the aligned grid
+// visits. Samples are below 2^31 and P <= 2^29, so indices fit unsigned 32 bits.
 
 // Walks (item, chunk) pairs of this CTA in order. T and nch are the current
 // item's frame's (from its descriptor in a batch, else from args); the writer
 // reads the rest when it needs it. kArith: the item is one (band, tile, gate)
-// over the frame, and its chunks are those that hold samples of the gate
-// (the current one c, the next one cn).
+// over the frame; c is then the chunk's first sample, at gate position pos.
 template <bool kFrames, bool kHold, bool kArith = false>
 struct Walk {
   int item, c, c0, f, bi, bj, c1, frame, T, nch, T0;
@@ -451,8 +419,8 @@ struct Walk {
   int mode, hold, fN, fresh, atomic;
   int64_t fB;
   int32_t* fvis;
-  // kArith: the gate of the current descriptor, and the item's next chunk
-  int gP, gphase, ga, gb, cn;
+  // kArith: the gate of the current descriptor, and the chunk's gate position
+  int gP, gphase, ga, gb, pos;
   __device__ __forceinline__ void load() {
     for (; item < nitems; item += stride) {
       const int4 w = items[item];
@@ -485,10 +453,12 @@ struct Walk {
         // a gated group covers all of its gate's samples in the frame, like a whole tile
         const bool whole = kHold || kArith || (w.z == 0 && w.w == nch);
         mode = atomic ? 2 : (whole ? (fresh ? 0 : 1) : 2);
-        if (kArith) {
-          c = gate_chunk(c, c1, T, gP, gphase, ga, gb);
-          if (c >= c1) continue;  // the gate has no samples here: nothing to do or write
-          cn = gate_chunk(c + 1, c1, T, gP, gphase, ga, gb);
+        if (kArith) {  // the gate's first sample
+          c = 0;
+          pos = gphase;
+          if (ga >= gb) continue;  // a gate without positions
+          if (pos < ga || pos >= gb) gate_run();
+          if (past_end(c)) continue;  // the gate has no samples here: nothing to do or write
         }
       } else {
         bj = w.y >> 16;
@@ -521,17 +491,32 @@ struct Walk {
     nch = a.nch;
     T0 = 0;
     c = -1;
-    c1 = cn = 0;
+    c1 = 0;
   }
   __device__ __forceinline__ bool valid() const { return item < nitems; }
   // the current chunk is the item's last
-  __device__ __forceinline__ bool last() const { return kArith ? cn >= c1 : c + 1 == c1; }
+  __device__ __forceinline__ bool last() const {
+    return kArith ? past_end(c + (gb - pos > kTC ? static_cast<uint32_t>(kTC) : gate_gap())) : c + 1 == c1;
+  }
+  // kArith: samples from here to the gate's next run, and the step there
+  __device__ __forceinline__ uint32_t gate_gap() const { return pos < ga ? ga - pos : gP - pos + ga; }
+  __device__ __forceinline__ bool past_end(uint32_t s) const { return s >= static_cast<uint32_t>(T); }
+  __device__ __forceinline__ void gate_run() {
+    c += gate_gap();
+    pos = ga;
+  }
+  // kArith: samples of the chunk
+  __device__ __forceinline__ int gate_rows() const { return min(min(kTC, gb - pos), T - c); }
   __device__ __forceinline__ void next() {
     if (kArith) {
-      if (cn < c1) {
-        c = cn;
-        cn = gate_chunk(c + 1, c1, T, gP, gphase, ga, gb);
-        return;
+      if (item >= 0) {  // (not before the first unit)
+        if (gb - pos > kTC) {
+          c += kTC;
+          pos += kTC;
+        } else {
+          gate_run();
+        }
+        if (!past_end(c)) return;
       }
     } else if (++c != c1) {
       return;
@@ -678,13 +663,8 @@ __global__ void __launch_bounds__(kThreads, 1) corr_tile_kernel(const __grid_con
         ChunkMeta& m = sm.meta[s];
         m.f = ld.f;
         m.bij = ld.bi | (ld.bj << 16);
-        if (kArith) {
-          gate_windows(ld.c, ld.T, ld.gP, ld.gphase, ld.ga, ld.gb, m);
-        } else {
-          m.lo = ld.T0 - ld.c * kTC;
-          m.hi = ld.T - ld.c * kTC;
-          m.lo2 = m.hi2 = 0;
-        }
+        m.lo = kArith ? 0 : ld.T0 - ld.c * kTC;
+        m.hi = kArith ? ld.gate_rows() : ld.T - ld.c * kTC;
         m.flags = kMetaValid | ((ld.last() && !ld.hold) ? kMetaEnd : 0) | (ld.mode << 4);
         m.N = ld.fN;
         m.B = ld.fB;
@@ -692,8 +672,9 @@ __global__ void __launch_bounds__(kThreads, 1) corr_tile_kernel(const __grid_con
       }
       // (the arrive releases the stores above to the slot's waiters)
       mbar_arrive_expect_tx(&sm.full[s], diag ? kBoxBytes : 2 * kBoxBytes);
-      tma_load_3d(sm.box[s][0], map, &sm.full[s], ld.bi * kTile, ld.f, ld.c * kTC);
-      if (!diag) tma_load_3d(sm.box[s][1], map, &sm.full[s], ld.bj * kTile, ld.f, ld.c * kTC);
+      const int t = kArith ? ld.c : ld.c * kTC;
+      tma_load_3d(sm.box[s][0], map, &sm.full[s], ld.bi * kTile, ld.f, t);
+      if (!diag) tma_load_3d(sm.box[s][1], map, &sm.full[s], ld.bj * kTile, ld.f, t);
       ++issued;
       ld.next();
     };
@@ -730,7 +711,7 @@ __global__ void __launch_bounds__(kThreads, 1) corr_tile_kernel(const __grid_con
           break;
         }
         const ChunkMeta& m = sm.meta[s];
-        const int flags = m.flags, bij = m.bij, lo = m.lo, hi = m.hi, lo2 = m.lo2, hi2 = m.hi2;
+        const int flags = m.flags, bij = m.bij, lo = m.lo, hi = m.hi;
         if (threadIdx.x == kMmaWarps * 32) sm.pmeta[buf] = m;  // passed on with the planes
         if (!(flags & kMetaValid)) {
           mbar_arrive(&sm.pfull[buf]);
@@ -747,7 +728,7 @@ __global__ void __launch_bounds__(kThreads, 1) corr_tile_kernel(const __grid_con
           if (lo <= 0 && hi >= kTC)
             unpack_unit<false, kEnc>(box, pl0, pl1, pl2, j == 1, eg, tg, p, 0, kTC);
           else
-            unpack_unit<true, kEnc>(box, pl0, pl1, pl2, j == 1, eg, tg, p, lo, hi, lo2, hi2);
+            unpack_unit<true, kEnc>(box, pl0, pl1, pl2, j == 1, eg, tg, p, lo, hi);
         }
         mbar_arrive(&sm.pfull[buf]);
         mbar_arrive(&sm.bempty[s]);
@@ -832,7 +813,7 @@ __global__ void __launch_bounds__(kThreads, 1) corr_tile_kernel(const __grid_con
       if (!(flags & kMetaValid)) return;  // end of this CTA's chunks
       const int bi = m.bij & 0xFFFF, bj = m.bij >> 16;
       // rows past the last valid one are masked to zero: their k-steps can be skipped
-      const int nvalid = m.hi2 > m.lo2 ? max(m.hi, m.hi2) : m.hi;
+      const int nvalid = m.hi;
       int pr, pc, sel;
       product_chunk<kEnc, kSplitT>(sm, buf, warp, lane, bi == bj, nvalid, args.hybrid, it, pr, pc, sel, acc);
       // the writer's fields, read before the buffer (and its metadata) is released

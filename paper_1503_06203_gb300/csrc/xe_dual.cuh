@@ -64,7 +64,7 @@ struct __align__(16) DualMeta {
   int32_t bij;    // bi | bj << 16
   int32_t rows;   // samples past this one count as zero
   int32_t f;      // band
-  int32_t lo, hi, lo2, hi2;  // masked chunks: valid samples [lo, hi) and [lo2, hi2)
+  int32_t lo, hi; // masked chunks: valid samples [lo, hi)
   int64_t B;
   int32_t* vis;
   int32_t N;
@@ -241,7 +241,7 @@ __device__ __forceinline__ void dp_step(uint32_t ra, uint32_t rb, DpFrag& n, con
     }
 }
 
-// Samples [first, 128) of the chunk's main product (planes ra, rb) into acc,
+// Samples [first, end) of the chunk's main product (planes ra, rb) into acc,
 // and `half` of them (from sq) of Q (planes qa, qb) into acq; then the next
 // chunk's first operands. Addresses carry the lane's row and swizzle; XOR with
 // a sample offset selects the samples. Loops of two steps (4.6 KB of code
@@ -249,13 +249,13 @@ __device__ __forceinline__ void dp_step(uint32_t ra, uint32_t rb, DpFrag& n, con
 // instruction cache, beyond which straight dp4a code runs 1.6x slower.
 template <bool kDiag, typename Wait, typename Addr>
 __device__ __forceinline__ void dp_chunk(uint32_t ra, uint32_t rb, uint32_t qa, uint32_t qb, uint32_t first,
-                                         uint32_t sq, uint32_t half, Wait next_chunk, Addr next_addr, DpFrag (&f)[2],
+                                         uint32_t end, uint32_t sq, uint32_t half, Wait next_chunk, Addr next_addr, DpFrag (&f)[2],
                                          int32_t (&acc)[8][8], int32_t (&acq)[8][8]) {
 #pragma unroll 1
-  for (uint32_t o = first; o < kTC; o += 16) {
+  for (uint32_t o = first; o < end; o += 16) {
     opaque(o);
     dp_step<kDiag>(ra ^ (o + 8), rb ^ (o + 8), f[1], f[0], acc);
-    const bool last = o + 16 == kTC;
+    const bool last = o + 16 == end;
     dp_step<kDiag>(last ? qa ^ sq : ra ^ (o + 16), last ? qb ^ sq : rb ^ (o + 16), f[0], f[1], acc);
   }
   next_chunk();
@@ -344,23 +344,17 @@ __global__ void __launch_bounds__(kDualThreads, 1) corr_dual_kernel(const __grid
         tensormap_acquire(map);
         fenced = map;
       }
-      ChunkMeta w;
-      if (kArith) {
-        gate_windows(ld.c, ld.T, ld.gP, ld.gphase, ld.ga, ld.gb, w);
-      } else {
-        w.lo = ld.T0 - ld.c * kTC;
-        w.hi = ld.T - ld.c * kTC;
-        w.lo2 = w.hi2 = 0;
-      }
-      const int rows = w.hi2 > w.lo2 ? max(w.hi, w.hi2) : w.hi;
-      const int mk = rows < kTC ? 2 : 2 + ((issued * kThreeOf8 >> 3) - ((issued - 1) * kThreeOf8 >> 3));
+      const int lo = kArith ? 0 : ld.T0 - ld.c * kTC;
+      const int rows = kArith ? ld.gate_rows() : ld.T - ld.c * kTC;
+      // k-steps of 32 samples that hold any; a full chunk alternates 2 and 3 on the tensor cores, a shorter
+      // one gives dp4a its last one if it has more than one
+      const int ksteps = (min(rows, kTC) + 31) >> 5;
+      const int mk = ksteps == 4 ? 2 + ((issued * kThreeOf8 >> 3) - ((issued - 1) * kThreeOf8 >> 3)) : max(1, ksteps - 1);
       int flags = kMetaValid | (mk << 8);
-      if (w.lo > 0 || w.hi < kTC) {
+      if (lo > 0 || rows < kTC) {
         flags |= kMetaMasked;
-        m.lo = w.lo;
-        m.hi = w.hi;
-        m.lo2 = w.lo2;
-        m.hi2 = w.hi2;
+        m.lo = lo;
+        m.hi = rows;
       }
       if (ld.last() && !(kHold && ld.hold)) {  // the item is written after this chunk
         if constexpr (kFrames) {
@@ -378,8 +372,9 @@ __global__ void __launch_bounds__(kDualThreads, 1) corr_dual_kernel(const __grid
       *reinterpret_cast<int4*>(&m) = make_int4(flags, ld.bi | (ld.bj << 16), rows, ld.f);
       // (the arrive releases the stores above to the slot's waiters)
       mbar_arrive_expect_tx(&sm.full[s], diag ? kBoxBytes : 2 * kBoxBytes);
-      tma_load_3d(sm.box[s][0], map, &sm.full[s], ld.bi * kTile, ld.f, ld.c * kTC);
-      if (!diag) tma_load_3d(sm.box[s][1], map, &sm.full[s], ld.bj * kTile, ld.f, ld.c * kTC);
+      const int t = kArith ? ld.c : ld.c * kTC;
+      tma_load_3d(sm.box[s][0], map, &sm.full[s], ld.bi * kTile, ld.f, t);
+      if (!diag) tma_load_3d(sm.box[s][1], map, &sm.full[s], ld.bj * kTile, ld.f, t);
     };
     if (producer) {
       if (!kFrames) tma_prefetch_desc(&tmap);
@@ -433,11 +428,11 @@ __global__ void __launch_bounds__(kDualThreads, 1) corr_dual_kernel(const __grid
       const bool diag = (bij & 0xFFFF) == (bij >> 16);
       // the dp4a samples of an off-diagonal tile's column side: the two words of every 8 samples swapped
       const int swap = !diag && uw >= (flags >> 8) ? 4 : 0;
-      if (flags & kMetaMasked) {  // rows outside both windows count as zero: blank the words this thread unpacks
-        const int lo = m.lo, hi = m.hi, lo2 = m.lo2, hi2 = m.hi2;
+      if (flags & kMetaMasked) {  // rows outside [lo, hi) count as zero: blank the words this thread unpacks
+        const int lo = m.lo, hi = m.hi;
 #pragma unroll 1
         for (int t = 16 * tg; t < 16 * tg + 16; ++t)
-          if (!((t >= lo && t < hi) || (t >= lo2 && t < hi2)))
+          if (t < lo || t >= hi)
             for (int j = 0; j < (diag ? 1 : 2); ++j)
               reinterpret_cast<uint32_t*>(sm.box[s][j])[t * (kTile / 4) + eg] = 0x88888888u;
         fence_proxy_async();  // before the slot's next copy
@@ -449,7 +444,7 @@ __global__ void __launch_bounds__(kDualThreads, 1) corr_dual_kernel(const __grid
         const uint32_t pld = smem_u32(sm.plane[buf][1][kPsd]);
         const int rx = p | (j ? swap : 0);
         uint32_t r[16];
-        unpack_load<false, false>(sm.box[s][j], eg, tg, rx, 0, kTC, 0, 0, r);
+        unpack_load<false, false>(sm.box[s][j], eg, tg, rx, 0, kTC, r);
         unpack_store<false>(r, pl, pl + kPlaneBytes, j ? 0u : pl + kPsd * kPlaneBytes, j || diag ? pld : 0u, eg, tg, rx);
       }
       __syncwarp();
@@ -598,7 +593,8 @@ __global__ void __launch_bounds__(kDualThreads, 1) corr_dual_kernel(const __grid
       ok = mbar_wait_bounded(&sm.pfull[nbuf], nphase, kSpinLimit);
       next_head = meta_head(sm.pmeta[nbuf]);
     };
-    const uint32_t first = 32 * (head.x >> 8), half = (kTC - first) / 2;
+    // samples [first, end), whole k-steps; Q's half of them
+    const uint32_t first = 32 * (head.x >> 8), end = min(kTC, (head.z + 31) & ~31), half = (end - first) / 2;
     if (head.z > static_cast<int>(first)) {
       if (!primed) dp_load(ra ^ first, rb ^ first, fr[0]);
       auto next_addr = [&](uint32_t& na, uint32_t& nb) {  // (if there is no next chunk, this one's: loaded, not used)
@@ -610,9 +606,9 @@ __global__ void __launch_bounds__(kDualThreads, 1) corr_dual_kernel(const __grid
         nb = (base + ob + (xdiag ? 0 : 3 * kPlaneBytes)) ^ o;
       };
       if (diag)
-        dp_chunk<true>(ra, rb, qa, qb, first, first + half * q, half, next_chunk, next_addr, fr, acc, acq);
+        dp_chunk<true>(ra, rb, qa, qb, first, end, first + half * q, half, next_chunk, next_addr, fr, acc, acq);
       else
-        dp_chunk<false>(ra, rb, qa, qb, first, first + half * q, half, next_chunk, next_addr, fr, acc, acq);
+        dp_chunk<false>(ra, rb, qa, qb, first, end, first + half * q, half, next_chunk, next_addr, fr, acc, acq);
       primed = 1;
     } else {
       next_chunk();

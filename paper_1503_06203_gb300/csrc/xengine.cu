@@ -76,7 +76,9 @@ int device_setup(int dev) {
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemBytes));
   for (const void* k : {reinterpret_cast<const void*>(xe::corr_dual_kernel<xe::kSingle>),
-                        reinterpret_cast<const void*>(xe::corr_dual_kernel<xe::kBatch>)}) {
+                        reinterpret_cast<const void*>(xe::corr_dual_kernel<xe::kBatch>),
+                        reinterpret_cast<const void*>(xe::corr_dual_kernel<xe::kGated>),
+                        reinterpret_cast<const void*>(xe::corr_dual_kernel<xe::kGateArith>)}) {
     // its register re-split draws on the registers it is launched with: fewer would leave it waiting for good
     cudaFuncAttributes at;
     e = cudaFuncGetAttributes(&at, k);
@@ -621,9 +623,8 @@ int grow_set(BatchSet& b, size_t frames, size_t items) {
   return CORR_OK;
 }
 
-// The correlator of a batched launch: the default share runs the dual-engine
-// kernel, every other one the runtime-split kernel (as 8 or 6). Gated launches
-// run the runtime-split kernel.
+// The correlator of a batched or gated launch: the default share runs the
+// dual-engine kernel, every other one the runtime-split kernel (as 8 or 6).
 struct CorrLaunch {
   void* fn;
   unsigned threads, smem;
@@ -631,7 +632,10 @@ struct CorrLaunch {
 
 CorrLaunch corr_launch_of(int mode, int hybrid) {
   if (hybrid == xe::kSplitDual)
-    return {reinterpret_cast<void*>(xe::corr_dual_kernel<xe::kBatch>), xe::kDualThreads, static_cast<unsigned>(kDualSmemBytes)};
+    return {mode == xe::kBatch   ? reinterpret_cast<void*>(xe::corr_dual_kernel<xe::kBatch>)
+            : mode == xe::kGated ? reinterpret_cast<void*>(xe::corr_dual_kernel<xe::kGated>)
+                                 : reinterpret_cast<void*>(xe::corr_dual_kernel<xe::kGateArith>),
+            xe::kDualThreads, static_cast<unsigned>(kDualSmemBytes)};
   return {mode == xe::kBatch   ? reinterpret_cast<void*>(xe::corr_tile_kernel<xe::kBatch, false>)
           : mode == xe::kGated ? reinterpret_cast<void*>(xe::corr_tile_kernel<xe::kGated, false>)
                                : reinterpret_cast<void*>(xe::corr_tile_kernel<xe::kGateArith, false>),
@@ -639,8 +643,8 @@ CorrLaunch corr_launch_of(int mode, int hybrid) {
 }
 
 // The split a batched or gated launch runs: the runtime-split kernel knows tensor cores only and 6 of 8.
-int shared_split(int hybrid, bool gated) {
-  return hybrid == xe::kSplitMma || (hybrid == xe::kSplitDual && !gated) ? hybrid : xe::kSplit6;
+int shared_split(int hybrid) {
+  return hybrid == xe::kSplitMma || hybrid == xe::kSplitDual ? hybrid : xe::kSplit6;
 }
 
 // kind: 1 = gate segments (corr_tile_kernel<kGated>), 2 = gate arithmetic (<kGateArith>).
@@ -1017,7 +1021,7 @@ static int batch_shared(corr_handle_t* const* hs, const uint8_t* const* inputs, 
     d.nb = static_cast<int32_t>(ceil_div(h->N, xe::kTile));
     d.per = static_cast<int32_t>(per[k]);
   }
-  const int hybrid = shared_split(chunk_hybrid_flag(hs[0]->product, hs[0]->mma_steps), false);
+  const int hybrid = shared_split(chunk_hybrid_flag(hs[0]->product, hs[0]->mma_steps));
   r.p_frames = reinterpret_cast<const xe::FrameDesc*>(r.d_blk);
   r.p_first = reinterpret_cast<const int64_t*>(r.d_blk + kFirstOff);
   r.p_order = reinterpret_cast<const int32_t*>(r.d_blk + kOrderOff);
@@ -1051,13 +1055,16 @@ static int batch_shared(corr_handle_t* const* hs, const uint8_t* const* inputs, 
 // ---- gated correlation, gate windows by arithmetic ---------------------------------
 // One descriptor per gate (the same frame map, the gate's accumulators and
 // fresh flag, the gate arithmetic), one item per (band, tile, gate) over the
-// whole frame; the kernel visits only the chunks that hold samples of the
-// item's gate and masks the other rows. Items are dealt round-robin in
+// whole frame; the kernel cuts the gate's runs of samples into chunks. Items are dealt round-robin in
 // (gate, band, tile) order.
 int gated_arith_launch(corr_handle_t* const* gates, int G, const CUtensorMap& map, int32_t T, int32_t period,
                        int32_t phase, const std::vector<int64_t>& per_gate, const std::vector<int32_t>& gate_fresh,
                        cudaStream_t st) {
   corr_handle* h0 = gates[0];
+  if (G == 1) {  // one run over the whole frame, not one a period
+    period = 1 << 29;
+    phase = 0;
+  }
   if (G >= kMaxBatchFrames) return fail(CORR_EINVAL, "gated: at most %d gates", kMaxBatchFrames - 1);
   std::vector<int32_t> bi, bj;
   triangle_tiles(h0->N, xe::kTile, bi, bj);
@@ -1112,7 +1119,7 @@ int gated_arith_launch(corr_handle_t* const* gates, int G, const CUtensorMap& ma
     d.G = G;
     d.gate = g;
   }
-  const int hybrid = shared_split(chunk_hybrid_flag(h0->product, h0->mma_steps), true);
+  const int hybrid = shared_split(chunk_hybrid_flag(h0->product, h0->mma_steps));
   if (!b.exec || b.key_frames != G || b.key_items != nitems || b.key_grid != grid || b.key_hybrid != hybrid ||
       b.key_gated != 2 || b.key_err != h0->d_err)
     if ((rc = build_graph(b, G, nitems, grid, h0->d_err, hybrid, 2))) return rc;
@@ -1274,7 +1281,7 @@ int gated_impl(corr_handle_t* const* gates, int G, const uint8_t* in, int32_t T,
     d.t0 = empty ? 1 : segs[s].t0;  // t0 > T: nothing is valid
     d.atomic = 0;
   }
-  const int hybrid = shared_split(chunk_hybrid_flag(h0->product, h0->mma_steps), true);
+  const int hybrid = shared_split(chunk_hybrid_flag(h0->product, h0->mma_steps));
   if (!b.exec || b.key_frames != nseg || b.key_items != nitems || b.key_grid != grid || b.key_hybrid != hybrid ||
       b.key_gated != 1 || b.key_err != h0->d_err)
     if ((rc = build_graph(b, nseg, nitems, grid, h0->d_err, hybrid, 1))) return rc;
