@@ -240,15 +240,22 @@ void frame_tiles(int32_t N, int32_t F, std::vector<int2>& tiles, std::vector<dou
 
 // Items of a frame: its first `whole` tiles over all chunks, the other tiles'
 // time axis cut into `ranges` ranges of whole chunks (range-major, each range
-// over those tiles in frame order). CTA k of P takes items k, k+P, ... so the
+// over those tiles in frame order). With diag_first the last `slots` whole
+// tiles are dealt diagonal ones (the cheaper ones) first, so that the CTAs
+// that take a range after them are those with time left. CTA k of P takes items k, k+P, ... so the
 // CTAs running together work on neighbouring tiles of one band over the same
 // time range and share its input in L2.
-void make_items(const std::vector<int2>& tiles, int64_t nch, int64_t whole, int64_t ranges, std::vector<int4>& items) {
+bool diagonal(const int2& t) { return (t.y & 0xFFFF) == (t.y >> 16); }
+
+void make_items(const std::vector<int2>& tiles, int64_t nch, int64_t slots, int64_t whole, int64_t ranges,
+                bool diag_first, std::vector<int4>& items) {
   items.clear();
   const int64_t n = static_cast<int64_t>(tiles.size());
   items.reserve(static_cast<size_t>(whole + (n - whole) * ranges));
   for (int64_t u = 0; u < whole; ++u) items.push_back(make_int4(tiles[u].x, tiles[u].y, 0, static_cast<int32_t>(nch)));
   if (whole == n) return;
+  if (diag_first && whole >= slots)
+    std::stable_partition(items.end() - slots, items.end(), [](const int4& w) { return diagonal(make_int2(w.x, w.y)); });
   const int64_t per = ceil_div(nch, ranges);
   for (int64_t c0 = 0; c0 < nch; c0 += per)
     for (int64_t u = whole; u < n; ++u)
@@ -259,6 +266,8 @@ void make_items(const std::vector<int2>& tiles, int64_t nch, int64_t whole, int6
 // Time of an item beside its chunks (filling its pipeline, merging the two
 // engines' sums, writing the tile), in chunks of an off-diagonal tile.
 constexpr double kItemCost = 0.8;
+// Zeroing the output that cut tiles add onto (a launch of its own), in chunks.
+constexpr double kCutCost = 1.0;
 
 // Pick the schedule: whole tiles only (no atomics), if that keeps the busiest
 // CTA within 3% of an even share; else the best of: as many whole tiles as
@@ -275,6 +284,7 @@ void plan_items(int32_t N, int32_t F, int32_t T, int64_t slots, std::vector<int4
   const int64_t ntiles = static_cast<int64_t>(tiles.size());
   const int64_t nch = ceil_div(T, xe::kTC);
   int64_t best_whole = ntiles, best_ranges = 1;
+  bool best_first = false;
   if (forced_split > 0) {
     best_ranges = std::min<int64_t>(forced_split, nch);
     best_whole = best_ranges > 1 ? 0 : ntiles;
@@ -283,7 +293,7 @@ void plan_items(int32_t N, int32_t F, int32_t T, int64_t slots, std::vector<int4
     for (double c : cost) total += c * static_cast<double>(nch) + kItemCost;
     std::vector<double> load(static_cast<size_t>(slots));
     // the busiest CTA's cost over an even share, items dealt round-robin
-    auto eff_of = [&](int64_t whole, int64_t ranges) {
+    auto eff_of = [&](int64_t whole, int64_t ranges, bool diag_first) {
       std::fill(load.begin(), load.end(), 0.0);
       const int64_t per = ceil_div(nch, ranges), rem = ntiles - whole;
       const int64_t P = std::min(slots, whole + rem * ceil_div(nch, per));
@@ -292,12 +302,15 @@ void plan_items(int32_t N, int32_t F, int32_t T, int64_t slots, std::vector<int4
         load[k] += c + kItemCost;
         if (++k == P) k = 0;
       };
-      for (int64_t u = 0; u < whole; ++u) deal(cost[u] * static_cast<double>(nch));
+      for (int64_t u = 0; u < whole - (diag_first ? slots : 0); ++u) deal(cost[u] * static_cast<double>(nch));
+      for (int diag = 1; diag_first && diag >= 0; --diag)  // (as make_items)
+        for (int64_t u = whole - slots; u < whole; ++u)
+          if (diagonal(tiles[u]) == (diag == 1)) deal(cost[u] * static_cast<double>(nch));
       for (int64_t c0 = 0; rem && c0 < nch; c0 += per)
         for (int64_t u = whole; u < ntiles; ++u) deal(cost[u] * static_cast<double>(std::min(per, nch - c0)));
-      return *std::max_element(load.begin(), load.end()) * static_cast<double>(slots) / total;
+      return (*std::max_element(load.begin(), load.end()) + (rem ? kCutCost : 0.0)) * static_cast<double>(slots) / total;
     };
-    double best = eff_of(ntiles, 1);
+    double best = eff_of(ntiles, 1, false);
     const int64_t full = ntiles / slots;
     for (int64_t a = full; best > 1.03 && a >= 0 && a >= full - 2; --a) {
       const int64_t whole = (a == full - 2 ? 0 : a) * slots, rem = ntiles - whole;
@@ -306,18 +319,44 @@ void plan_items(int32_t N, int32_t F, int32_t T, int64_t slots, std::vector<int4
       for (int64_t k = 1; k <= 2; ++k) ranges.push_back(std::min<int64_t>(64, k * slots / rem));
       for (int64_t r : ranges) {
         if (r < 2 || r > nch || rem * r > std::max<int64_t>(4 * slots, 2 * rem)) continue;
-        const double eff = eff_of(whole, r);
-        if (eff < best - 1e-9) {
-          best = eff;
-          best_whole = whole;
-          best_ranges = r;
+        for (int first = 0; first <= (whole ? 1 : 0); ++first) {
+          const double eff = eff_of(whole, r, first);
+          if (eff < best - 1e-9) {
+            best = eff;
+            best_whole = whole;
+            best_ranges = r;
+            best_first = first;
+          }
         }
       }
     }
   }
-  make_items(tiles, nch, best_whole, best_ranges, items);
+  make_items(tiles, nch, slots, best_whole, best_ranges, best_first, items);
   *split_out = best_whole == ntiles ? 1 : best_ranges;
   *grid_out = std::min<int64_t>(slots, static_cast<int64_t>(items.size()));
+}
+
+// The same choice by the items' number alone (every tile counted as an
+// off-diagonal one), for a caller that schedules on every call: whole tiles
+// for whole rounds of the CTAs (or none), the others cut into `ranges`.
+void quick_split(int64_t ntiles, int64_t nch, int64_t slots, int64_t max_items, int64_t* whole, int64_t* ranges) {
+  *whole = ntiles;
+  *ranges = 1;
+  double best = static_cast<double>(ceil_div(ntiles, slots)) * (static_cast<double>(nch) + kItemCost);
+  for (int64_t w : {ntiles / slots * slots, int64_t(0)}) {
+    const int64_t rem = ntiles - w;
+    if (rem == 0) continue;
+    for (int64_t r : {2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64}) {
+      if (r > nch || w + rem * r > max_items) break;
+      const double t = static_cast<double>(w / slots) * (static_cast<double>(nch) + kItemCost) + kCutCost +
+                       static_cast<double>(ceil_div(rem * r, slots)) * (static_cast<double>(ceil_div(nch, r)) + kItemCost);
+      if (t < best) {
+        best = t;
+        *whole = w;
+        *ranges = r;
+      }
+    }
+  }
 }
 
 // Schedule a frame of T samples for the resident CTAs of this device.
@@ -1802,14 +1841,17 @@ static __device__ __align__(256) int4 g_noalloc_scratch[1 + kNoAllocMaxItems];
 std::mutex g_noalloc_mu;
 int4* g_noalloc_addr[64];  // device address of g_noalloc_scratch, per device
 
-// Writes the frame's work list: item k = split s, tile u of the frame (bands
-// outermost, each band's upper triangle row by row), chunks [s*per, ...).
-__global__ void noalloc_plan_kernel(int4* items, int32_t nb, int32_t F, int32_t nch, int32_t per, int64_t nitems) {
+// Writes the frame's work list: item k < whole is tile k (bands outermost,
+// each band's upper triangle row by row) over all chunks; the other tiles are
+// cut into ranges of `per` chunks, range by range.
+__global__ void noalloc_plan_kernel(int4* items, int32_t nb, int32_t F, int32_t nch, int32_t per, int64_t whole,
+                                    int64_t nitems) {
   const int64_t per_band = static_cast<int64_t>(nb) * (nb + 1) / 2;
-  const int64_t ntiles = per_band * F;
+  const int64_t rem = per_band * F - whole;
   for (int64_t k = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; k < nitems;
        k += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int64_t s = k / ntiles, u = k % ntiles;
+    const bool cut = k >= whole;
+    const int64_t s = cut ? (k - whole) / rem : 0, u = cut ? whole + (k - whole) % rem : k;
     const int32_t f = static_cast<int32_t>(u / per_band);
     int64_t q = u % per_band;
     int32_t bi = 0;
@@ -1819,7 +1861,7 @@ __global__ void noalloc_plan_kernel(int4* items, int32_t nb, int32_t F, int32_t 
     }
     const int32_t bj = bi + static_cast<int32_t>(q);
     const int32_t c0 = static_cast<int32_t>(s * per);
-    const int32_t c1 = static_cast<int32_t>(min(static_cast<int64_t>(nch), (s + 1) * per));
+    const int32_t c1 = cut ? static_cast<int32_t>(min(static_cast<int64_t>(nch), (s + 1) * per)) : nch;
     items[k] = make_int4(f, bi | (bj << 16), c0, c1);
   }
 }
@@ -1860,22 +1902,22 @@ extern "C" int corr_correlate_noalloc(const uint8_t* packed_dev, int32_t N, int3
   int4* scratch = nullptr;
   if ((rc = noalloc_setup(dev, &scratch))) return rc;
   const int64_t slots = static_cast<int64_t>(g_sms[dev]) * g_blocks_per_sm[dev];
-  // time split: enough items to keep every CTA busy, within the array and the frame's chunks
-  int64_t split = std::min<int64_t>({ceil_div(4 * slots, ntiles), kNoAllocMaxItems / ntiles, nch, int64_t(64)});
-  split = std::max<int64_t>(split, 1);
+  // whole tiles, or cut ones where those leave CTAs idle, within the array and the frame's chunks
+  int64_t whole, split;
+  quick_split(ntiles, nch, slots, kNoAllocMaxItems, &whole, &split);
   const int64_t per = ceil_div(nch, split);
   split = ceil_div(nch, per);  // no empty ranges
-  const int64_t nitems = ntiles * split;
+  const int64_t nitems = whole + (ntiles - whole) * split;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t vis_bytes = static_cast<size_t>(F) * (static_cast<size_t>(N) * (N + 1) / 2) * 2 * sizeof(int32_t);
   // the fault word starts at zero; time-split items add atomically onto a zeroed output
   if ((e = cudaMemsetAsync(scratch, 0, sizeof(int4), st)) != cudaSuccess)
     return fail(CORR_ECUDA, "noalloc: clearing the fault word: %s", cudaGetErrorString(e));
-  if (split > 1 && (e = cudaMemsetAsync(vis_dev, 0, vis_bytes, st)) != cudaSuccess)
+  if (whole < ntiles && (e = cudaMemsetAsync(vis_dev, 0, vis_bytes, st)) != cudaSuccess)
     return fail(CORR_ECUDA, "noalloc: clearing the output: %s", cudaGetErrorString(e));
   const int pb = static_cast<int>(std::min<int64_t>(ceil_div(nitems, 256), 1024));
   noalloc_plan_kernel<<<pb, 256, 0, st>>>(scratch + 1, static_cast<int32_t>(nb), F, static_cast<int32_t>(nch),
-                                          static_cast<int32_t>(per), nitems);
+                                          static_cast<int32_t>(per), whole, nitems);
   if ((e = cudaGetLastError()) != cudaSuccess) return fail(CORR_ECUDA, "noalloc plan: %s", cudaGetErrorString(e));
   CUtensorMap tm;
   if ((rc = make_tmap(&tm, packed_dev, N, F, T))) return rc;
