@@ -855,16 +855,45 @@ __global__ void __launch_bounds__(kThreads, 1) corr_tile_kernel(const __grid_con
 
 // Copy the bands [f0, f0 + F) of a frame [T][F_in][N] whose rows are not
 // 16-byte aligned into an aligned staging buffer [T][F][Np] (Np = N rounded
-// up to 16); padding bytes are 0x88. rows = T * F.
-__global__ void repack_rows_kernel(const uint8_t* __restrict__ src, uint8_t* __restrict__ dst, int64_t rows,
-                                   int32_t N, int32_t Np, int32_t F, int32_t F_in, int32_t f0) {
-  const int64_t total = rows * Np;
-  for (int64_t k = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; k < total;
-       k += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int64_t r = k / Np;
-    const int32_t e = static_cast<int32_t>(k - r * Np);
-    const int64_t t = r / F, f = r - t * F;
-    dst[k] = e < N ? src[(t * F_in + f0 + f) * N + e] : static_cast<uint8_t>(0x88);
+// up to 16); padding bytes are 0x88. rows = T * F; a block copies `per` rows
+// (per * Np near 32 KB). HBM-bound: a thread makes 16 bytes from the up to
+// five aligned words that hold them, so a warp moves 512 bytes with whole
+// words; byte by byte, with a 64-bit division each, the copy took longer than
+// the correlation it prepares. A word is read only if it holds a byte of the
+// row, so it lies in the same page as that byte.
+constexpr int kRepackThreads = 256;
+
+__global__ void __launch_bounds__(kRepackThreads) repack_rows_kernel(const uint8_t* __restrict__ src,
+                                                                     uint8_t* __restrict__ dst, int64_t rows,
+                                                                     int32_t per, int32_t N, int32_t Np, int32_t F,
+                                                                     int32_t F_in, int32_t f0) {
+  const int64_t r0 = static_cast<int64_t>(blockIdx.x) * per;
+  const uint32_t n = static_cast<uint32_t>(min(static_cast<int64_t>(per), rows - r0));
+  const uint32_t quads = static_cast<uint32_t>(Np) >> 4;
+  const int64_t t0 = r0 / F;
+  const uint32_t fr = static_cast<uint32_t>(r0 - t0 * F);
+#pragma unroll 4
+  for (uint32_t k = threadIdx.x; k < n * quads; k += kRepackThreads) {
+    const uint32_t r = k / quads, e0 = 16 * (k - r * quads);
+    int64_t row = r0 + r;  // row of the source frame
+    if (F != F_in) {
+      const uint32_t t = (fr + r) / static_cast<uint32_t>(F);
+      row = (t0 + t) * F_in + f0 + (fr + r - t * F);
+    }
+    const uintptr_t a = reinterpret_cast<uintptr_t>(src) + static_cast<uintptr_t>(row * N + e0);
+    const uint32_t* w = reinterpret_cast<const uint32_t*>(a & ~static_cast<uintptr_t>(3));
+    const int off = static_cast<int>(a & 3), live = min(16, N - static_cast<int>(e0));  // bytes of the row here
+    uint32_t v[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) v[i] = 4 * i < live + off ? __ldg(w + i) : 0u;
+    uint32_t o[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int b = live - 4 * i;  // live bytes of this word
+      const uint32_t mask = b >= 4 ? 0xFFFFFFFFu : b <= 0 ? 0u : (1u << (8 * b)) - 1u;
+      o[i] = (__funnelshift_r(v[i], v[i + 1], 8 * off) & mask) | (0x88888888u & ~mask);
+    }
+    *reinterpret_cast<uint4*>(dst + (r0 + r) * Np + e0) = make_uint4(o[0], o[1], o[2], o[3]);
   }
 }
 

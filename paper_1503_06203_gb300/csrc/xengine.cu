@@ -576,11 +576,11 @@ int stage_if_needed(corr_handle* h, const uint8_t* in, int32_t T, cudaStream_t s
     h->stage_bytes = need;
   }
   const int64_t rows = static_cast<int64_t>(T) * h->F;
-  const int64_t total = rows * np;
-  const int threads = 256;
-  const int64_t blocks = std::min<int64_t>(ceil_div(total, threads), int64_t(g_sms[h->device]) * 8);
-  xe::repack_rows_kernel<<<static_cast<int>(std::max<int64_t>(blocks, 1)), threads, 0, st>>>(
-      in, h->stage, rows, h->N, np, h->F, h->F_in, h->f0);
+  const int32_t per = std::max(1, 32768 / np);
+  const int64_t blocks = ceil_div(rows, per);
+  if (blocks > INT32_MAX) return fail(CORR_EINVAL, "frame too large to stage");
+  xe::repack_rows_kernel<<<static_cast<int>(blocks), xe::kRepackThreads, 0, st>>>(in, h->stage, rows, per, h->N, np, h->F,
+                                                                                h->F_in, h->f0);
   XE_CHECK(h, cudaGetLastError());
   ++h->launches;
   *frame = h->stage;
