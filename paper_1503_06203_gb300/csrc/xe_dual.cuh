@@ -49,10 +49,12 @@ constexpr int kDualDpWarps = 4;
 constexpr int kDualUnpackWarp = kDualMmaWarps + kDualDpWarps;
 constexpr int kDualThreads = (kDualUnpackWarp + 4) * 32;
 // Of every 8 chunks, those whose first 96 samples run on the tensor cores and
-// the last 32 on dp4a (the others: 64 and 64). Measured at 0, 1, 2, 3 and 4:
-// N=8192 2172, 2118, 2046, 2014 and 2079 us, N=256 1223, 1192, 1162, 1137 and
-// 1172 us (F=1, T=2048 and F=64, T=16384).
-constexpr uint32_t kThreeOf8 = 3;
+// the last 32 on dp4a (the others: 64 and 64), off and on the diagonal.
+// Measured at 0, 1, 2, 3 and 4 off it: N=8192 2172, 2118, 2046, 2014 and 2079
+// us (F=1, T=2048). On it (where dp4a skips more of the tile than the MMA's
+// granularity lets the tensor cores skip) at 0, 1, 2 and 3: N=64 224, 214, 218
+// and 224 us (F=152, T=16384), N=256 662, 654, 655 and 660 us (F=152, T=4096).
+constexpr uint32_t kThreeOff = 3, kThreeDiag = 1;
 constexpr int kRegsLaunch = 128, kRegsMma = 96, kRegsDp = 216, kRegsUnpack = 104;
 static_assert(2 * kRegsMma + kRegsDp + kRegsUnpack <= 4 * kRegsLaunch, "setmaxnreg draws on the launch's registers");
 
@@ -349,7 +351,8 @@ __global__ void __launch_bounds__(kDualThreads, 1) corr_dual_kernel(const __grid
       // k-steps of 32 samples that hold any; a full chunk alternates 2 and 3 on the tensor cores, a shorter
       // one gives dp4a its last one if it has more than one
       const int ksteps = (min(rows, kTC) + 31) >> 5;
-      const int mk = ksteps == 4 ? 2 + ((issued * kThreeOf8 >> 3) - ((issued - 1) * kThreeOf8 >> 3)) : max(1, ksteps - 1);
+      const uint32_t three = diag ? kThreeDiag : kThreeOff;
+      const int mk = ksteps == 4 ? 2 + ((issued * three >> 3) - ((issued - 1) * three >> 3)) : max(1, ksteps - 1);
       int flags = kMetaValid | (mk << 8);
       if (lo > 0 || rows < kTC) {
         flags |= kMetaMasked;
