@@ -317,6 +317,10 @@ __global__ void __launch_bounds__(kDualThreads, 1) corr_dual_kernel(const __grid
     fence_barrier_init();
   }
   for (int k = threadIdx.x; k < 2 * kTile * kTile; k += kDualThreads) sm.part[0][k] = 0;
+  // The next launch may set its CTAs up as these leave their SMs; a launch that
+  // was allowed to do so waits here for everything before it in its stream.
+  launch_dependents();
+  wait_prerequisites();
   __syncthreads();
 
   if (warp >= kDualUnpackWarp) {

@@ -429,6 +429,23 @@ int check_handle(corr_handle* h) {
   return CORR_OK;
 }
 
+// The dual-engine kernel on one frame, as a dependent launch: a frame behind
+// another one sets its CTAs up (and is launched at all) while the other's last
+// CTAs run, and waits inside for it to finish before touching memory.
+cudaError_t launch_dual(int32_t grid, cudaStream_t st, const CUtensorMap& tm, const xe::CorrArgs& a) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(grid));
+  cfg.blockDim = dim3(xe::kDualThreads);
+  cfg.dynamicSmemBytes = kDualSmemBytes;
+  cfg.stream = st;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, xe::corr_dual_kernel<xe::kSingle>, tm, a);
+}
+
 // Launch the correlator over the handle's F bands of Np bytes (16-byte
 // aligned rows) at `frame`, time samples row_bytes apart.
 int launch_frame(corr_handle* h, const uint8_t* frame, int32_t Np, int64_t row_bytes, const Plan& pl,
@@ -478,7 +495,7 @@ int launch_frame(corr_handle* h, const uint8_t* frame, int32_t Np, int64_t row_b
   else if (a.hybrid == xe::kSplit7)
     xe::corr_tile_kernel<xe::kSingle, false, xe::kSplit7><<<pl.grid, xe::kThreads, kSmemBytes, st>>>(tm, a);
   else if (a.hybrid == xe::kSplitDual)
-    xe::corr_dual_kernel<xe::kSingle><<<pl.grid, xe::kDualThreads, kDualSmemBytes, st>>>(tm, a);
+    XE_CHECK(h, launch_dual(pl.grid, st, tm, a));
   else if (a.hybrid == xe::kSplit4)
     xe::corr_tile_kernel<xe::kSingle, false, xe::kSplit4><<<pl.grid, xe::kThreads, kSmemBytes, st>>>(tm, a);
   else
