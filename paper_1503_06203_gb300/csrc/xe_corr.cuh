@@ -108,13 +108,16 @@ struct __align__(128) CorrSmem {
 };
 
 // Swizzle of a plane (rows of kTC = 128 bytes, 8 chunks of 16): chunk c of
-// row e sits at chunk c ^ (e & 7). Eight consecutive rows then hit eight
-// different 16-byte bank groups (ldmatrix, the dp4a operand loads), rows 8
-// apart share their swizzle (so a lane's rows are immediate offsets from one
-// address), and the unpack stores below (rows 4eg + slot across a
-// quarter-warp) are free of conflicts through their slot order.
+// row e sits at chunk c ^ f(e), f(e) = the three low bits of e rotated. Eight
+// consecutive rows then hit eight different 16-byte bank groups (ldmatrix, the
+// dp4a operand loads), rows 8 apart share their swizzle (so a lane's rows are
+// immediate offsets from one address), and the unpack stores are free of
+// conflicts: here rows 4eg + slot across a quarter-warp, through their slot
+// order; in the dual-engine kernel two rows x four chunks (f of an even row and
+// of the next differ by 4).
+__device__ __forceinline__ constexpr int plane_swz(int e) { return ((e & 1) << 2) | ((e >> 1) & 3); }
 __device__ __forceinline__ uint32_t plane_off(int e, int chunk) {
-  return static_cast<uint32_t>(e * kTC + ((chunk ^ (e & 7)) << 4));
+  return static_cast<uint32_t>(e * kTC + ((chunk ^ plane_swz(e)) << 4));
 }
 
 // ---- unpack: packed box [time][element] -> planes [element][time] --------------
@@ -126,37 +129,63 @@ __device__ __forceinline__ uint32_t plane_off(int e, int chunk) {
 //   v - 8      = (v + 0x78) ^ 0x80
 //   hi + lo - 16 = (hi + lo + 0x70) ^ 0x80      (xr + xi)
 //   hi - lo    = ((hi | 0x80) - lo) ^ 0x80       (xr - xi)
-// Rows are loaded in the order k ^ rx, with bit 0 of rx set for lanes 16..31,
+// Rows are loaded in the order k ^ p, with p set for lanes 16..31,
 // and element quad eg stores its elements in the order slot ^ (eg >> 1 & 3),
 // so that loads and stores are free of bank conflicts; runtime prmt selectors
-// undo both reorderings. Bit 2 of rx (a multiple of four rows, so the
-// selectors do not see it) leaves the two words of every 8 samples swapped in
-// the planes.
+// undo both reorderings.
 //
 // kEnc (offset-encoded operands, the Eq. 3 route): the planes keep the
 // encoded nibbles, all unsigned: Xr = hi, Xi = lo, Xr + Xi = hi + lo (row
 // side) and Xr - Xi + 15 = (hi + 15) - lo (column side), each in [0, 30];
 // masked rows are 0x00, which zeroes every product they enter (each product
 // has a row-side factor Xr, Xi or Xr + Xi).
-//
-// pl0, pl1, pls, pld: the planes xr, xi, xr + xi and xr - xi (0 = not wanted).
+
+// One 16-byte vector of each plane (element's row offset `off` in it) from the
+// packed samples wd: pl0, pl1, pls, pld: the planes xr, xi, xr + xi and
+// xr - xi (0 = not wanted).
+template <bool kEnc>
+__device__ __forceinline__ void unpack_vec(const uint32_t (&wd)[4], uint32_t off, uint32_t pl0, uint32_t pl1,
+                                           uint32_t pls, uint32_t pld) {
+  uint32_t hi[4], lo[4], v[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    hi[j] = (wd[j] >> 4) & 0x0F0F0F0Fu;
+    lo[j] = wd[j] & 0x0F0F0F0Fu;
+  }
+  if (pls) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = kEnc ? hi[j] + lo[j] : (hi[j] + lo[j] + 0x70707070u) ^ 0x80808080u;
+    sts128(pls + off, v[0], v[1], v[2], v[3]);
+  }
+  if (pld) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      v[j] = kEnc ? (hi[j] + 0x0F0F0F0Fu) - lo[j] : ((hi[j] | 0x80808080u) - lo[j]) ^ 0x80808080u;
+    sts128(pld + off, v[0], v[1], v[2], v[3]);
+  }
+  if (pl0) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (!kEnc) hi[j] = (hi[j] + 0x78787878u) ^ 0x80808080u;
+      if (!kEnc) lo[j] = (lo[j] + 0x78787878u) ^ 0x80808080u;
+    }
+    sts128(pl0 + off, hi[0], hi[1], hi[2], hi[3]);
+    sts128(pl1 + off, lo[0], lo[1], lo[2], lo[3]);
+  }
+}
+
 template <bool kMasked, bool kEnc>
-__device__ __forceinline__ void unpack_load(const uint8_t* box, int eg, int tg, int rx, int lo, int hi,
-                                            uint32_t (&r)[16]) {
+__device__ __forceinline__ void unpack_unit(const uint8_t* box, uint32_t pl0, uint32_t pl1, uint32_t pl2,
+                                            bool side_b, int eg, int tg, int p, int lo, int hi) {
   const uint32_t* w = reinterpret_cast<const uint32_t*>(box);
+  uint32_t r[16];
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
-    const int t = 16 * tg + (k ^ rx);
+    const int t = 16 * tg + (k ^ p);
     r[k] = w[t * (kTile / 4) + eg];
     // rows outside [lo, hi): no products
     if (kMasked) r[k] = (t >= lo && t < hi) ? r[k] : (kEnc ? 0u : 0x88888888u);
   }
-}
-
-template <bool kEnc>
-__device__ __forceinline__ void unpack_store(const uint32_t (&r)[16], uint32_t pl0, uint32_t pl1, uint32_t pls,
-                                             uint32_t pld, int eg, int tg, int rx) {
-  const int p = rx & 1;
   const int s = (eg >> 1) & 3;
   const uint32_t sel01 = p ? 0x1504u : 0x5140u;  // interleave two rows, bytes 0-1
   const uint32_t sel23 = p ? 0x3726u : 0x7362u;  // bytes 2-3
@@ -177,44 +206,8 @@ __device__ __forceinline__ void unpack_store(const uint32_t (&r)[16], uint32_t p
     wd[3][j] = prmt(x1, y1, hi16);
   }
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int e = 4 * eg + (k ^ s);
-    const uint32_t off = plane_off(e, tg);
-    uint32_t hi[4], lo[4], v[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      hi[j] = (wd[k][j] >> 4) & 0x0F0F0F0Fu;
-      lo[j] = wd[k][j] & 0x0F0F0F0Fu;
-    }
-    if (pls) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) v[j] = kEnc ? hi[j] + lo[j] : (hi[j] + lo[j] + 0x70707070u) ^ 0x80808080u;
-      sts128(pls + off, v[0], v[1], v[2], v[3]);
-    }
-    if (pld) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        v[j] = kEnc ? (hi[j] + 0x0F0F0F0Fu) - lo[j] : ((hi[j] | 0x80808080u) - lo[j]) ^ 0x80808080u;
-      sts128(pld + off, v[0], v[1], v[2], v[3]);
-    }
-    if (pl0) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if (!kEnc) hi[j] = (hi[j] + 0x78787878u) ^ 0x80808080u;
-        if (!kEnc) lo[j] = (lo[j] + 0x78787878u) ^ 0x80808080u;
-      }
-      sts128(pl0 + off, hi[0], hi[1], hi[2], hi[3]);
-      sts128(pl1 + off, lo[0], lo[1], lo[2], lo[3]);
-    }
-  }
-}
-
-template <bool kMasked, bool kEnc>
-__device__ __forceinline__ void unpack_unit(const uint8_t* box, uint32_t pl0, uint32_t pl1, uint32_t pl2,
-                                            bool side_b, int eg, int tg, int rx, int lo, int hi) {
-  uint32_t r[16];
-  unpack_load<kMasked, kEnc>(box, eg, tg, rx, lo, hi, r);
-  unpack_store<kEnc>(r, pl0, pl1, side_b ? 0u : pl2, side_b ? pl2 : 0u, eg, tg, rx);
+  for (int k = 0; k < 4; ++k)
+    unpack_vec<kEnc>(wd[k], plane_off(4 * eg + (k ^ s), tg), pl0, pl1, side_b ? 0u : pl2, side_b ? pl2 : 0u);
 }
 
 // ---- product: one 128-sample chunk of a warp's 16 x 16 piece of the tile --------

@@ -23,7 +23,7 @@
 // N=8192, F=4, T=2048 9451 -> 8180 us; N=1024, F=64, T=4096 4735 -> 4102 us.
 //
 // Roles (512 threads, one CTA per SM, launched with 128 registers a thread,
-// then re-split by setmaxnreg: 2 x 96 + 216 + 104 = 512 a lane):
+// then re-split by setmaxnreg: 2 x 104 + 216 + 88 = 512 a lane):
 //   warps 0-7   tensor cores: the first 64 or 96 samples of each chunk, P1, P2
 //               and Q of a 32 x 16 piece each (48 sums), two warps per
 //               sub-partition (one cannot hide its own fragment loads: 80
@@ -33,7 +33,14 @@
 //               over its samples, and Q over half of them, so the four warps
 //               carry equal work with two 8 x 8 micro-tiles of sums each (128
 //               registers), operands double-buffered 8 samples ahead;
-//   warps 12-15 TMA issue and unpack (as in xe_corr.cuh).
+//   warps 12-15 TMA issue and unpack. ldmatrix transposes the bytes (sm_103a's
+//               16 x 16 byte form), so a 16-byte vector of samples of an
+//               element takes half a load instruction and no byte permutes:
+//               about 180 instructions a warp and box, where loading row words
+//               and permuting took 230. Every one of them delays the dp4a warp
+//               that shares its issue port: N=8192 (F=1, T=2048) 2009 -> 1939
+//               us, N=256 (F=152, T=4096) 654 -> 638 us with the shares below
+//               re-tuned.
 // At the end of an item the dp4a warps fold their sums into (Re, Im) parts and
 // add them into a tile in shared memory; the tensor warps add theirs and write
 // the packed triangle from it, in whole 128-byte runs of a row.
@@ -50,12 +57,12 @@ constexpr int kDualUnpackWarp = kDualMmaWarps + kDualDpWarps;
 constexpr int kDualThreads = (kDualUnpackWarp + 4) * 32;
 // Of every 8 chunks, those whose first 96 samples run on the tensor cores and
 // the last 32 on dp4a (the others: 64 and 64), off and on the diagonal.
-// Measured at 0, 1, 2, 3 and 4 off it: N=8192 2172, 2118, 2046, 2014 and 2079
-// us (F=1, T=2048). On it (where dp4a skips more of the tile than the MMA's
-// granularity lets the tensor cores skip) at 0, 1, 2 and 3: N=64 224, 214, 218
-// and 224 us (F=152, T=16384), N=256 662, 654, 655 and 660 us (F=152, T=4096).
-constexpr uint32_t kThreeOff = 3, kThreeDiag = 1;
-constexpr int kRegsLaunch = 128, kRegsMma = 96, kRegsDp = 216, kRegsUnpack = 104;
+// Measured at 1, 2, 3 and 4 off it: N=8192 2001, 1939, 1977 and 2046 us (F=1,
+// T=2048). On it (where dp4a skips more of the tile than the MMA's granularity
+// lets the tensor cores skip) at 0, 1 and 2: N=64 213, 206 and 211 us (F=152,
+// T=16384), N=256 646, 638 and 638 us (F=152, T=4096).
+constexpr uint32_t kThreeOff = 2, kThreeDiag = 1;
+constexpr int kRegsLaunch = 128, kRegsMma = 104, kRegsDp = 216, kRegsUnpack = 88;
 static_assert(2 * kRegsMma + kRegsDp + kRegsUnpack <= 4 * kRegsLaunch, "setmaxnreg draws on the launch's registers");
 
 // What the roles need to know of a chunk: written by the TMA issuer beside the
@@ -73,8 +80,11 @@ struct __align__(16) DualMeta {
 };
 enum : int { kMetaMasked = 8 };
 
+// (1024: the boxes' TMA swizzle follows the address)
+constexpr uint32_t kDualAlign = 1024;
+
 struct __align__(128) DualSmem {
-  uint8_t box[kDualStages][2][kBoxBytes];          // TMA ring: [stage][A|B][time][element]
+  uint8_t box[kDualStages][2][kBoxBytes];          // TMA ring: [stage][A|B][time][element], 64-byte swizzle
   uint8_t plane[kDualBufs][2][3][kPlaneBytes];     // [buffer][A|B][slot][element][time]
   int32_t part[2][kTile * kTile];                  // Re and Im of the item under way, swizzled (part_at)
   uint64_t full[kDualStages], bempty[kDualStages]; // box landed / read by the 4 unpack warps
@@ -300,7 +310,8 @@ __global__ void __launch_bounds__(kDualThreads, 1) corr_dual_kernel(const __grid
   constexpr bool kArith = kMode == kGateArith;
   extern __shared__ uint8_t smem_raw[];
   // (aligned by an offset from smem_raw, so that the compiler keeps shared-space accesses)
-  DualSmem& sm = *reinterpret_cast<DualSmem*>(smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u));
+  DualSmem& sm =
+      *reinterpret_cast<DualSmem*>(smem_raw + ((kDualAlign - smem_u32(smem_raw) % kDualAlign) % kDualAlign));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
@@ -328,7 +339,18 @@ __global__ void __launch_bounds__(kDualThreads, 1) corr_dual_kernel(const __grid
     regs_down<kRegsUnpack>();
     const int uw = warp - kDualUnpackWarp;  // 0..3
     const bool producer = uw == 0 && lane == 0;
-    const int eg = lane & 15, p = lane >> 4, tg = 2 * uw + p;  // samples 16tg..16tg+15 of each chunk
+    // The transpose is ldmatrix's: warp uw takes elements 16 uw .. + 15 of a box, and lane 4 g + q, from
+    // four matrices of 16 samples (quads 16 q + 4 b .. + 3 as rows 4 q .. 4 q + 3 of matrix b), the 16
+    // samples 16 q .. + 15 of elements g and g + 8, for samples 0..63 and 64..127. A row address is a
+    // lane's own, so a quad pair that the planes hold swapped is read swapped (row_off[1]).
+    const int row = lane & 15, bl = lane >> 4, rq = row >> 2;
+    uint32_t row_off[2];
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      const int t = 16 * rq + 4 * (bl ^ x) + (row & 3);
+      row_off[x] = static_cast<uint32_t>(t * kTile + ((uw ^ ((t >> 1) & 3)) << 4));
+    }
+    const uint32_t out = (16 * uw + (lane >> 2)) * kTC + (((lane & 3) ^ plane_swz(lane >> 2)) << 4);
     Walk<kFrames, kHold, kArith> ld;
     uint32_t issued = 0;
     const CUtensorMap* fenced = nullptr;
@@ -433,26 +455,32 @@ __global__ void __launch_bounds__(kDualThreads, 1) corr_dual_kernel(const __grid
         break;
       }
       const bool diag = (bij & 0xFFFF) == (bij >> 16);
-      // the dp4a samples of an off-diagonal tile's column side: the two words of every 8 samples swapped
-      const int swap = !diag && uw >= (flags >> 8) ? 4 : 0;
-      if (flags & kMetaMasked) {  // rows outside [lo, hi) count as zero: blank the words this thread unpacks
+      if (flags & kMetaMasked) {  // rows outside [lo, hi) count as zero: blank what this warp unpacks of them
         const int lo = m.lo, hi = m.hi;
 #pragma unroll 1
-        for (int t = 16 * tg; t < 16 * tg + 16; ++t)
+        for (int t = lane; t < kTC; t += 32)
           if (t < lo || t >= hi)
             for (int j = 0; j < (diag ? 1 : 2); ++j)
-              reinterpret_cast<uint32_t*>(sm.box[s][j])[t * (kTile / 4) + eg] = 0x88888888u;
+              *reinterpret_cast<uint4*>(sm.box[s][j] + t * kTile + ((uw ^ ((t >> 1) & 3)) << 4)) =
+                  make_uint4(0x88888888u, 0x88888888u, 0x88888888u, 0x88888888u);
+        __syncwarp();
         fence_proxy_async();  // before the slot's next copy
       }
       // a diagonal tile's column side is its row side, so its xr - xi comes from the same pass
 #pragma unroll 1
       for (int j = 0; j < (diag ? 1 : 2); ++j) {
-        const uint32_t pl = smem_u32(sm.plane[buf][j][0]);
-        const uint32_t pld = smem_u32(sm.plane[buf][1][kPsd]);
-        const int rx = p | (j ? swap : 0);
-        uint32_t r[16];
-        unpack_load<false, false>(sm.box[s][j], eg, tg, rx, 0, kTC, r);
-        unpack_store<false>(r, pl, pl + kPlaneBytes, j ? 0u : pl + kPsd * kPlaneBytes, j || diag ? pld : 0u, eg, tg, rx);
+        const uint32_t box = smem_u32(sm.box[s][j]), pl = smem_u32(sm.plane[buf][j][0]);
+        const uint32_t pld = j || diag ? smem_u32(sm.plane[buf][1][kPsd]) : 0u, pls = j ? 0u : pl + kPsd * kPlaneBytes;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {  // samples 64 h .. 64 h + 63
+          // the dp4a samples of an off-diagonal tile's column side: the two words of every 8 samples swapped
+          const uint32_t at = box + (j && 2 * h + (rq >> 1) >= (flags >> 8) ? row_off[1] : row_off[0]) + 4096 * h;
+          uint32_t wd[2][4];
+          ldsm_t8_x2(at, wd[0][0], wd[1][0], wd[0][1], wd[1][1]);
+          ldsm_t8_x2(at + 512, wd[0][2], wd[1][2], wd[0][3], wd[1][3]);
+#pragma unroll
+          for (int e = 0; e < 2; ++e) unpack_vec<false>(wd[e], (out ^ (64 * h)) + 1024 * e, pl, pl + kPlaneBytes, pls, pld);
+        }
       }
       __syncwarp();
       if (lane == 0) {
@@ -488,8 +516,8 @@ __global__ void __launch_bounds__(kDualThreads, 1) corr_dual_kernel(const __grid
 #pragma unroll
     for (int k = 0; k < 48; ++k) (&acc[0][0][0][0])[k] = 0;
     const int l7 = lane & 7;
-    const uint32_t xa = static_cast<uint32_t>((lane >> 4) ^ l7) << 4;        // A: k half = lane / 16
-    const uint32_t xb = static_cast<uint32_t>(((lane >> 3) & 1) ^ l7) << 4;  // B: k half = (lane / 8) & 1
+    const uint32_t xa = static_cast<uint32_t>((lane >> 4) ^ plane_swz(l7)) << 4;        // A: k half = lane / 16
+    const uint32_t xb = static_cast<uint32_t>(((lane >> 3) & 1) ^ plane_swz(l7)) << 4;  // B: k half = (lane / 8) & 1
     const uint32_t arow = (lane & 15) * kTC + xa, brow = (l7 + ((lane >> 4) << 3)) * kTC + xb;
     int dr, dc;
     diag_piece(warp, dr, dc);
@@ -571,7 +599,7 @@ __global__ void __launch_bounds__(kDualThreads, 1) corr_dual_kernel(const __grid
   uint32_t clear = 1;  // the next chunk begins an item
   const int q = (warp >> 1) & 1, h = warp & 1;
   const int lr = lane >> 2, lc = 4 * h + (lane & 3);
-  const uint32_t oa = lr * kTC + (lr << 4), ob = lc * kTC + (lc << 4);
+  const uint32_t oa = lr * kTC + (plane_swz(lr) << 4), ob = lc * kTC + (plane_swz(lc) << 4);
   DpFrag fr[2];
   if (!mbar_wait_bounded(&sm.pfull[0], 0, kSpinLimit)) {
     if (lane == 0) atomicOr(args.err, kErrTimeoutFull);

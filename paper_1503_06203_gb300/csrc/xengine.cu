@@ -54,7 +54,7 @@ EncodeTiledFn encode_fn() {
 
 // ---- per-device kernel set-up ---------------------------------------------------
 constexpr size_t kSmemBytes = sizeof(xe::CorrSmem) + 128;  // + alignment slack
-constexpr size_t kDualSmemBytes = sizeof(xe::DualSmem) + 128;
+constexpr size_t kDualSmemBytes = sizeof(xe::DualSmem) + xe::kDualAlign;
 static_assert(kSmemBytes <= 232448 && kDualSmemBytes <= 232448, "shared memory of one CTA");
 std::mutex g_dev_mu;
 int g_blocks_per_sm[64];
@@ -385,11 +385,13 @@ void free_plan(Plan* pl) {
   *pl = Plan();
 }
 
+// swizzled: 16-byte pieces of a 64-byte box row are exchanged by a pattern of the
+// row (the dual-engine kernel's boxes).
 // 3-D map (elements, bands, time) of F bands of Np bytes starting at `base`;
 // consecutive time samples are row_bytes apart (0: F * Np, a frame of exactly
 // these bands). Elements past Np and samples past T read as zero bytes.
 int make_tmap(CUtensorMap* m, const uint8_t* base, int32_t Np, int32_t F, int32_t T, uint32_t box_n = xe::kTile,
-              uint32_t box_t = xe::kTC, int64_t row_bytes = 0) {
+              uint32_t box_t = xe::kTC, int64_t row_bytes = 0, bool swizzled = false) {
   EncodeTiledFn enc = encode_fn();
   if (!enc) return fail(CORR_ECUDA, "cuTensorMapEncodeTiled is not available from the driver");
   if (row_bytes == 0) row_bytes = static_cast<int64_t>(Np) * F;
@@ -398,7 +400,8 @@ int make_tmap(CUtensorMap* m, const uint8_t* base, int32_t Np, int32_t F, int32_
   cuuint32_t box[3] = {static_cast<cuuint32_t>(box_n), 1u, static_cast<cuuint32_t>(box_t)};
   cuuint32_t estr[3] = {1u, 1u, 1u};
   CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<uint8_t*>(base), dims, strides, box, estr,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, swizzled ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return fail(CORR_ECUDA, "cuTensorMapEncodeTiled failed (%d)", static_cast<int>(r));
   return CORR_OK;
@@ -451,9 +454,10 @@ cudaError_t launch_dual(int32_t grid, cudaStream_t st, const CUtensorMap& tm, co
 int launch_frame(corr_handle* h, const uint8_t* frame, int32_t Np, int64_t row_bytes, const Plan& pl,
                  cudaStream_t st) {
   CUtensorMap tm;
-  int rc = make_tmap(&tm, frame, Np, h->F, pl.T, xe::kTile, xe::kTC, row_bytes);
-  if (rc) return rc;
   const bool enc = effective_product(h->product) == 2;
+  const int hybrid = chunk_hybrid_flag(h->product, h->mma_steps);
+  int rc = make_tmap(&tm, frame, Np, h->F, pl.T, xe::kTile, xe::kTC, row_bytes, !enc && hybrid == xe::kSplitDual);
+  if (rc) return rc;
   if (enc) {
     // Eq. 3 route: nibble sums over this launch's samples, then the offset
     // terms stored (fresh) or added into the accumulators; the correlator
@@ -488,7 +492,7 @@ int launch_frame(corr_handle* h, const uint8_t* frame, int32_t Np, int64_t row_b
   a.B = h->B;
   a.vis = h->acc;
   a.fresh = h->fresh ? 1 : 0;
-  a.hybrid = chunk_hybrid_flag(h->product, h->mma_steps);
+  a.hybrid = hybrid;
   a.err = h->d_err;
   if (enc)  // (the offset-encoded route splits 96 / 32 or runs tensor cores only)
     xe::corr_tile_kernel<xe::kSingle, true><<<pl.grid, xe::kThreads, kSmemBytes, st>>>(tm, a);
@@ -1028,6 +1032,8 @@ static int batch_shared(corr_handle_t* const* hs, const uint8_t* const* inputs, 
   for (int k = 0; k < n; ++k) order[k] = k;
   std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) { return per[a] > per[b]; });
 
+  const int hybrid = shared_split(chunk_hybrid_flag(hs[0]->product, hs[0]->mma_steps));
+
   std::lock_guard<std::mutex> lk(g_batch_mu);
   if (!g_ring[dev]) g_ring[dev] = new (std::nothrow) BatchRing;
   if (!g_ring[dev]) return fail(CORR_ENOMEM, "batch ring");
@@ -1060,7 +1066,7 @@ static int batch_shared(corr_handle_t* const* hs, const uint8_t* const* inputs, 
     int64_t row_bytes;
     if ((rc = stage_if_needed(h, inputs[k], Tk, st, &frame, &np, &row_bytes))) return rc;
     xe::FrameDesc& d = desc[k];
-    if ((rc = make_tmap(&d.map, frame, np, h->F, Tk, xe::kTile, xe::kTC, row_bytes))) return rc;
+    if ((rc = make_tmap(&d.map, frame, np, h->F, Tk, xe::kTile, xe::kTC, row_bytes, hybrid == xe::kSplitDual))) return rc;
     if (ranges[k] > 1 && h->fresh) {  // time-split items add atomically onto zeros
       XE_CHECK(h, cudaMemsetAsync(h->acc, 0, static_cast<size_t>(h->F) * h->B * 2 * sizeof(int32_t), st));
       h->fresh = false;
@@ -1077,7 +1083,6 @@ static int batch_shared(corr_handle_t* const* hs, const uint8_t* const* inputs, 
     d.nb = static_cast<int32_t>(ceil_div(h->N, xe::kTile));
     d.per = static_cast<int32_t>(per[k]);
   }
-  const int hybrid = shared_split(chunk_hybrid_flag(hs[0]->product, hs[0]->mma_steps));
   r.p_frames = reinterpret_cast<const xe::FrameDesc*>(r.d_blk);
   r.p_first = reinterpret_cast<const int64_t*>(r.d_blk + kFirstOff);
   r.p_order = reinterpret_cast<const int32_t*>(r.d_blk + kOrderOff);
@@ -1113,7 +1118,7 @@ static int batch_shared(corr_handle_t* const* hs, const uint8_t* const* inputs, 
 // fresh flag, the gate arithmetic), one item per (band, tile, gate) over the
 // whole frame; the kernel cuts the gate's runs of samples into chunks. Items are dealt round-robin in
 // (gate, band, tile) order.
-int gated_arith_launch(corr_handle_t* const* gates, int G, const CUtensorMap& map, int32_t T, int32_t period,
+int gated_arith_launch(corr_handle_t* const* gates, int G, const CUtensorMap& map, int hybrid, int32_t T, int32_t period,
                        int32_t phase, const std::vector<int64_t>& per_gate, const std::vector<int32_t>& gate_fresh,
                        cudaStream_t st) {
   corr_handle* h0 = gates[0];
@@ -1175,7 +1180,6 @@ int gated_arith_launch(corr_handle_t* const* gates, int G, const CUtensorMap& ma
     d.G = G;
     d.gate = g;
   }
-  const int hybrid = shared_split(chunk_hybrid_flag(h0->product, h0->mma_steps));
   if (!b.exec || b.key_frames != G || b.key_items != nitems || b.key_grid != grid || b.key_hybrid != hybrid ||
       b.key_gated != 2 || b.key_err != h0->d_err)
     if ((rc = build_graph(b, G, nitems, grid, h0->d_err, hybrid, 2))) return rc;
@@ -1246,7 +1250,8 @@ int gated_impl(corr_handle_t* const* gates, int G, const uint8_t* in, int32_t T,
   int64_t row_bytes;
   if ((rc = stage_if_needed(h0, in, T, st, &frame, &np, &row_bytes))) return rc;
   CUtensorMap map;
-  if ((rc = make_tmap(&map, frame, np, h0->F, T, xe::kTile, xe::kTC, row_bytes))) return rc;
+  const int hybrid = shared_split(chunk_hybrid_flag(h0->product, h0->mma_steps));
+  if ((rc = make_tmap(&map, frame, np, h0->F, T, xe::kTile, xe::kTC, row_bytes, hybrid == xe::kSplitDual))) return rc;
   // Each (band, tile, gate) group is written once, by one CTA, with every
   // sample of its gate in this frame: stored into a fresh gate, added into
   // one that holds sums; no atomics. A gate with no samples here stays as it is.
@@ -1255,7 +1260,7 @@ int gated_impl(corr_handle_t* const* gates, int G, const uint8_t* in, int32_t T,
     gate_fresh[g] = gates[g]->fresh ? 1 : 0;
     if (per_gate[g] > 0) gates[g]->fresh = false;
   }
-  if (arith) return gated_arith_launch(gates, G, map, T, period, phase, per_gate, gate_fresh, st);
+  if (arith) return gated_arith_launch(gates, G, map, hybrid, T, period, phase, per_gate, gate_fresh, st);
   // groups: one (band, tile, gate) with all its segments in time order, run by
   // one CTA back to back ("hold" between them) and written once. Groups are
   // dealt in (band, gate, tile) order, each onto the least-loaded CTA: CTAs
@@ -1337,7 +1342,6 @@ int gated_impl(corr_handle_t* const* gates, int G, const uint8_t* in, int32_t T,
     d.t0 = empty ? 1 : segs[s].t0;  // t0 > T: nothing is valid
     d.atomic = 0;
   }
-  const int hybrid = shared_split(chunk_hybrid_flag(h0->product, h0->mma_steps));
   if (!b.exec || b.key_frames != nseg || b.key_items != nitems || b.key_grid != grid || b.key_hybrid != hybrid ||
       b.key_gated != 1 || b.key_err != h0->d_err)
     if ((rc = build_graph(b, nseg, nitems, grid, h0->d_err, hybrid, 1))) return rc;
@@ -1937,7 +1941,7 @@ extern "C" int corr_correlate_noalloc(const uint8_t* packed_dev, int32_t N, int3
                                           static_cast<int32_t>(per), whole, nitems);
   if ((e = cudaGetLastError()) != cudaSuccess) return fail(CORR_ECUDA, "noalloc plan: %s", cudaGetErrorString(e));
   CUtensorMap tm;
-  if ((rc = make_tmap(&tm, packed_dev, N, F, T))) return rc;
+  if ((rc = make_tmap(&tm, packed_dev, N, F, T, xe::kTile, xe::kTC, 0, true))) return rc;
   xe::CorrArgs a;
   a.items = scratch + 1;
   a.nitems = static_cast<int32_t>(nitems);
