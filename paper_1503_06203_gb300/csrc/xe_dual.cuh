@@ -599,7 +599,12 @@ __global__ void __launch_bounds__(kDualThreads, 1) corr_dual_kernel(const __grid
   uint32_t clear = 1;  // the next chunk begins an item
   const int q = (warp >> 1) & 1, h = warp & 1;
   const int lr = lane >> 2, lc = 4 * h + (lane & 3);
-  const uint32_t oa = lr * kTC + (plane_swz(lr) << 4), ob = lc * kTC + (plane_swz(lc) << 4);
+  // offsets of the lane's first row and column within a buffer's planes: main product and Q
+  constexpr uint32_t kSide = 3 * kPlaneBytes, kBuf = 2 * kSide;
+  const uint32_t ca = lr * kTC + (plane_swz(lr) << 4) + q * kPlaneBytes, cb = lc * kTC + (plane_swz(lc) << 4) + q * kPlaneBytes;
+  const uint32_t cq = (kPsd - q) * kPlaneBytes;
+  const uint32_t plane0 = smem_u32(sm.plane[0][0][0]);
+  uint32_t base = plane0;
   DpFrag fr[2];
   if (!mbar_wait_bounded(&sm.pfull[0], 0, kSpinLimit)) {
     if (lane == 0) atomicOr(args.err, kErrTimeoutFull);
@@ -611,10 +616,9 @@ __global__ void __launch_bounds__(kDualThreads, 1) corr_dual_kernel(const __grid
     const bool diag = (head.y & 0xFFFF) == (head.y >> 16);
     const int nbuf = buf + 1 == kDualBufs ? 0 : buf + 1;
     const uint32_t nphase = nbuf ? phase : phase ^ 1;
-    const uint32_t ap = smem_u32(sm.plane[buf][0][0]) + oa, bp = smem_u32(sm.plane[buf][1][0]) + ob;
-    const uint32_t ap_diag = smem_u32(sm.plane[buf][0][0]) + ob;
-    const uint32_t ra = ap + q * kPlaneBytes, rb = (diag ? ap_diag : bp) + q * kPlaneBytes;
-    const uint32_t qa = ap + kPsd * kPlaneBytes, qb = bp + kPsd * kPlaneBytes;
+    const uint32_t nbase = nbuf ? base + kBuf : plane0;
+    const uint32_t ra = base + ca, rb = base + cb + (diag ? 0u : kSide);
+    const uint32_t qa = ra + cq, qb = base + cb + kSide + cq;
     bool ok = true;
     opaque(clear);
     opaque(primed);
@@ -635,10 +639,9 @@ __global__ void __launch_bounds__(kDualThreads, 1) corr_dual_kernel(const __grid
       auto next_addr = [&](uint32_t& na, uint32_t& nb) {  // (if there is no next chunk, this one's: loaded, not used)
         const bool valid = next_head.x & kMetaValid;
         const bool xdiag = valid && (next_head.y & 0xFFFF) == (next_head.y >> 16);
-        const uint32_t base = smem_u32(sm.plane[valid ? nbuf : buf][0][0]) + q * kPlaneBytes;
-        const uint32_t o = 32 * (next_head.x >> 8);
-        na = (base + oa) ^ o;
-        nb = (base + ob + (xdiag ? 0 : 3 * kPlaneBytes)) ^ o;
+        const uint32_t at = valid ? nbase : base, o = 32 * (next_head.x >> 8);
+        na = (at + ca) ^ o;
+        nb = (at + cb + (xdiag ? 0u : kSide)) ^ o;
       };
       if (diag)
         dp_chunk<true>(ra, rb, qa, qb, first, end, first + half * q, half, next_chunk, next_addr, fr, acc, acq);
@@ -668,6 +671,7 @@ __global__ void __launch_bounds__(kDualThreads, 1) corr_dual_kernel(const __grid
     }
     head = next_head;
     buf = nbuf;
+    base = nbase;
     phase = nphase;
   }
 }
