@@ -49,8 +49,8 @@ WORKLOADS = {
     "large_n": ("LARGE_N", "large N: N=8192 F=4 T=2048, sigma=2.5 plus a common tone, one frame per launch"),
 }
 EXTRA_WORKLOADS = ("batched", "batched_small", "served", "lags_gates")
-KERNEL_NAME = "corr_tile_kernel"
-KERNEL_SOURCES = ["paper_1503_06203_gb300/csrc/xe_corr.cuh", "paper_1503_06203_gb300/csrc/xe_ptx.cuh"]
+KERNEL_SOURCES = ["paper_1503_06203_gb300/csrc/xe_dual.cuh", "paper_1503_06203_gb300/csrc/xe_corr.cuh",
+                  "paper_1503_06203_gb300/csrc/xe_ptx.cuh"]
 TRAFFIC_FILES = {"pathfinder": os.path.join(ROOT, "profiles", "corr_tile_kernel_pathfinder.md"),
                  "large_n": os.path.join(ROOT, "profiles", "corr_tile_kernel_large_n.md")}
 MEASURED_PEAKS = os.path.join(ROOT, "MEASURED_PEAKS.json")
@@ -174,10 +174,10 @@ def recorded_traffic(workload: str, product: int, split: int, mma_steps: int):
 def hardware_ops(N: int, F: int, T: int) -> float:
     """Tensor-core operations one launch issues (2 per int8 multiply-add).
 
-    64x64 tiles of 2x2 warps of 32x32; each warp runs 2x4 m16n8k32 MMAs per
-    product per 32 samples, three products (P1, P2, Q). On diagonal tiles the
-    warp below the diagonal is idle and the two on it skip 2 of 8 sub-tiles:
-    20 of 32 sub-tiles run.
+    A 64x64 tile is 32 sub-tiles of 16x8, one m16n8k32 MMA each per product
+    and 32 samples, three products (P1, P2, Q); on diagonal tiles 20 of them
+    run. Samples that dp4a takes are counted alike (on a diagonal tile it
+    computes 18 sub-tiles' worth).
     """
     nb = -(-N // 64)
     off, diag = nb * (nb - 1) // 2, nb
@@ -502,7 +502,7 @@ def single_frame_record(args, wl_key, frame, peaks, rank=0, world=1, bands=None,
                              "executes 6 integer operations per complex MAC, so achieved/peak can reach 4/3; "
                              "hw_frac compares the executed operations with the peak",
                      "hw_ops_per_launch": hw_ops, "hw_tops": round(hw_tops, 3), "hw_frac": round(hw_tops / peak, 4),
-                     "kernel": KERNEL_NAME, "avg_launch_ms": round(avg_kernel_ms, 4),
+                     "kernel": "corr_dual_kernel" if product == 1 and mma_steps == 5 else "corr_tile_kernel", "avg_launch_ms": round(avg_kernel_ms, 4),
                      "algorithmic_bytes": in_bytes + out_bytes,
                      "hbm_frac": round((in_bytes + out_bytes) / (avg_kernel_ms * 1e-3) / 1e9 / hbm, 4)},
         "e2e": {"value": round((job_ops or world * ops) * args.e2e_steps / (e2e_ms * 1e-3) / 1e12, 3), "unit": "TOPS",

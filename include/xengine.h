@@ -222,13 +222,14 @@ int corr_shift_lags(const uint8_t* in_dev, uint8_t* out_dev, int32_t N, int32_t 
  *   CORR_OPT_MMA_STEPS: for product paths 1 and 2, how many of every 8
  *     k-steps of 32 samples (two 128-sample chunks) run on the tensor cores,
  *     the rest on dp4a. 5 (the default) is, on product path 1, the kernel whose
- *     warps each drive one of the two pipes (64/64 and 96/32 in turn, 4.75 of
- *     8). The others run both pipes in every product warp: 8 = tensor cores
- *     only, 7 (chunks alternate 128/0 and 96/32), 6 (96/32 in every chunk), 4
- *     (64/64 off the diagonal, 96/32 on tiles with bi == bj). Single-frame
- *     calls (corr_accumulate, corr_accumulate_host) on product path 1 take
- *     every share; batched calls take 8, 6 or 5, gated calls and product path
- *     2 take 8 or 6 (other values run as 6).
+ *     warps each drive one of the two pipes: 64/64, with 96/32 in two of every
+ *     8 chunks (one on tiles with bi == bj). The others run both pipes in every
+ *     product warp: 8 = tensor cores only, 7 (chunks alternate 128/0 and
+ *     96/32), 6 (96/32 in every chunk), 4 (64/64 off the diagonal, 96/32 on
+ *     tiles with bi == bj). Single-frame calls (corr_accumulate,
+ *     corr_accumulate_host) on product path 1 take every share; batched and
+ *     gated calls take 8, 6 or 5 and product path 2 takes 8 or 6 (other values
+ *     run as 6).
  * A batched launch takes its product path and share from its first handle.
  * Returns CORR_OK, CORR_EINVAL or CORR_EBUSY.
  */

@@ -4,8 +4,9 @@ Knobs (results never depend on them; see corr_set_option in include/xengine.h):
 the product path (tensor cores + dp4a, tensor cores alone, or tensor cores +
 dp4a on offset-encoded operands with the Eq. 3 corrections), the share of
 each pair of 128-sample chunks that runs on the tensor cores (8, 7, 6, 5 or 4
-of 8 k-steps of 32 samples, the rest on dp4a; each share is its own kernel
-instantiation, built in), and the time split (automatic, or a fixed number
+of 8 k-steps of 32 samples, the rest on dp4a; 5 is the kernel with a warp
+group per pipe, the others are instantiations of the kernel that runs both
+pipes in every product warp), and the time split (automatic, or a fixed number
 of ranges). For a frame shape (N, F, T)
 the tuner times every candidate with CUDA events on random frames and keeps
 the choice in a JSON cache keyed by the GPU and the shape, so a shape is
@@ -39,7 +40,7 @@ def gpu_key() -> str:
     return f"{p.name}|sm_{p.major}{p.minor}|{p.multi_processor_count}sm"
 
 
-TUNER_VERSION = 2  # the candidate set and the kernels it chose among: entries of another version are not reused
+TUNER_VERSION = 3  # the candidate set and the kernels it chose among: entries of another version are not reused
 
 
 def shape_key(N: int, F: int, T: int) -> str:

@@ -1,10 +1,12 @@
-// The correlator kernel: TMA-staged 4-bit input, excess-8 unpack into
-// K-major int8 planes in shared memory, integer tensor-core Hermitian
-// product in the three-product form, packed upper-triangle writer.
+// The correlator kernel of product paths 0 and 2 and of the shares other than
+// the default (which xe_dual.cuh runs), and what both kernels share: TMA-staged
+// 4-bit input, excess-8 unpack into K-major int8 planes in shared memory,
+// integer Hermitian product in the three-product form, packed upper-triangle
+// writer.
 //
-// A CTA walks a contiguous range of (tile, time-chunk) units of one frame.
-// Tiles are 64x64 blocks (block row bi <= block column bj) of one band;
-// tiles below the diagonal are never scheduled (Sec. II.C, Fig. 1).
+// Work items are (band, tile, chunk range); tiles are 64x64 blocks (block row
+// bi <= block column bj) of one band; tiles below the diagonal are never
+// scheduled (Sec. II.C, Fig. 1).
 //
 // Arithmetic. Eq. 1 gives Re = sum xr_i xr_j + xi_i xi_j and
 // Im = sum xi_i xr_j - xr_i xi_j. With three real products per pair,

@@ -948,11 +948,10 @@ static int accumulate_alone(corr_handle_t* h, const uint8_t* packed_dev, int32_t
 }
 
 // Whole tiles per CTA slot from which a frame runs alone: its tiles then fill
-// every SM four times over, so it gains nothing from sharing a launch, and the
-// single-frame kernel (no frame descriptors or chunk metadata, tensor-core
-// share 5 built) runs it faster than the batched one. A frame of fewer
-// samples than its handle's T (a time piece) runs alone only where the
-// handle's schedule keeps tiles whole, so that every item stays balanced.
+// every SM four times over, so it gains nothing from sharing a launch, and a
+// launch of its own reads no frame descriptors. A frame of fewer samples than
+// its handle's T (a time piece) runs alone only where the handle's schedule
+// keeps tiles whole, so that every item stays balanced.
 constexpr int64_t kAloneWaves = CORR_BATCH_ALONE_WAVES;
 
 int batch_impl(corr_handle_t* const* hs, const uint8_t* const* inputs, const int32_t* Ts, int n, void* stream) {

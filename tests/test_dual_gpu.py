@@ -25,6 +25,7 @@ def xe():
     (60, 1, 97), (64, 1, 127), (128, 1, 128), (127, 2, 129), (129, 1, 160), (200, 1, 128 * 9 + 70), (64, 1, 128 * 17),
     (192, 300, 40),   # more whole tiles than CTAs, one short chunk each
     (256, 16, 1024),  # whole tiles and time-split ones in one launch
+    (20, 1, 128 * 513 + 70), (16, 1, 200000),  # long integrations
 ])
 @pytest.mark.parametrize("extreme", [False, True])
 def test_dual_kernel_matches_oracle(xe, N, F, T, extreme):
