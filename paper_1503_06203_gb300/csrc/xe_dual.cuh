@@ -5,22 +5,22 @@
 // cycle and sub-partition) and run side by side, so each takes about half of
 // every 128-sample chunk of a 64 x 64 tile. What bounds a kernel that uses
 // both is neither pipe but what feeds them:
-// - Shared memory. Every operand byte a warp loads costs the same on the data
-//   path whether its lanes share it or not, so the bytes per product fall only
-//   with the entries a thread owns. One warp running both pipes on a 16 x 16
-//   piece (chunk_hybrid in xe_corr.cuh: 96 registers, 24 of them sums) loads 6
-//   words per 8 dp4a; here a dp4a thread owns an 8 x 8 micro-tile of one
-//   product (16 words per 64 dp4a) and an MMA warp a 32 x 16 piece, which is
-//   what the register split below is for.
+// - Operand loads. One warp running both pipes on a 16 x 16 piece
+//   (chunk_hybrid in xe_corr.cuh: 96 registers, 24 of them sums) loads 6 words
+//   per 8 dp4a and keeps the shared-memory data path 77% busy; here a dp4a
+//   thread owns an 8 x 8 micro-tile of one product (16 words per 64 dp4a) and
+//   an MMA warp a 32 x 16 piece (55% busy), which is what the register split
+//   below is for.
 // - Instruction fetch. Straight dp4a code runs at full rate from loops of up to
 //   32 KB (the SM's instruction cache, all roles together) and 1.6x slower
 //   beyond; the first form of this kernel, unrolled to 137 KB, was slower than
 //   the kernel it replaces. So the loops below stay rolled.
 // - Issue slots: an int8 MMA takes 5 and a chunk's unpack about 500 a warp.
 //
-// Measured against the kernel that ran both pipes in every product warp (same
-// schedule): N=256, F=256, T=16384 5014 -> 4434 us (220 -> 249 effective TOPS);
-// N=8192, F=4, T=2048 9451 -> 8180 us; N=1024, F=64, T=4096 4735 -> 4102 us.
+// Measured against the kernel that ran both pipes in every product warp, whole
+// passes: N=256, F=256, T=16384 5017 -> 4222 us (220 -> 261 effective TOPS);
+// N=8192, F=4, T=2048 9439 -> 7974 us; N=1024, F=64, T=4096 4738 -> 3984 us
+// (schedules the same). Now: tensor pipe 79%, dp4a's pipe 63%, issue 62%.
 //
 // Roles (512 threads, one CTA per SM, launched with 128 registers a thread,
 // then re-split by setmaxnreg: 2 x 104 + 216 + 88 = 512 a lane):
@@ -132,8 +132,8 @@ __device__ __forceinline__ void mma_load(uint32_t pa, uint32_t pb, const MmaPiec
   if (kDiag && single) ldsm_x2(pb + (p.b1 ^ kx), f.b1[0], f.b1[1]);
 }
 
-// k-steps [0, ks) of the chunk. The other warp of the
-// sub-partition covers the fragment loads' latency.
+// k-steps [0, ks) of the chunk. The other warp of the sub-partition covers the
+// fragment loads' latency.
 template <bool kDiag>
 __device__ __forceinline__ void mma_chunk(uint32_t a_base, uint32_t b01, uint32_t b2, const MmaPiece& p, int ks,
                                           bool single, int32_t (&acc)[3][2][2][4]) {
@@ -190,6 +190,9 @@ __device__ __forceinline__ void add_subtile(int32_t* part, int row0, int col0, i
 // else add (red: the same result, and nothing to wait for, whether or not
 // other CTAs add to the tile). Entries with i > j or outside the N x N matrix
 // are dropped; entry (i, j) lives at (p(i, j)) * 2, p(i, j) = i N - i(i-1)/2 + j - i.
+// Lanes past ncol (a diagonal tile's 16 x 8 piece) touch nothing: their columns
+// are another warp's or past `part`. One branch for the read and the zeroing;
+// clamping the column instead took 1944 against 1934 us (N=8192, F=1, T=2048).
 __device__ __forceinline__ void write_rows(int32_t* part, int N, int32_t* band, int i0, int j0, int row0, int col0,
                                            int ncol, int lane, bool store) {
   const int col = col0 + (lane >> 1), j = j0 + col;
@@ -199,12 +202,14 @@ __device__ __forceinline__ void write_rows(int32_t* part, int N, int32_t* band, 
   const bool live = (lane >> 1) < ncol && j < N;
 #pragma unroll 1
   for (int r0 = 0; r0 < 16; r0 += 8) {
-    int32_t v[8];
+    int32_t v[8] = {};
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
       int32_t* s = src + part_at(row0 + r0 + r, col);
-      v[r] = *s;
-      if ((lane >> 1) < ncol) *s = 0;
+      if ((lane >> 1) < ncol) {
+        v[r] = *s;
+        *s = 0;
+      }
     }
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
@@ -261,8 +266,8 @@ __device__ __forceinline__ void dp_step(uint32_t ra, uint32_t rb, DpFrag& n, con
 // instruction cache, beyond which straight dp4a code runs 1.6x slower.
 template <bool kDiag, typename Wait, typename Addr>
 __device__ __forceinline__ void dp_chunk(uint32_t ra, uint32_t rb, uint32_t qa, uint32_t qb, uint32_t first,
-                                         uint32_t end, uint32_t sq, uint32_t half, Wait next_chunk, Addr next_addr, DpFrag (&f)[2],
-                                         int32_t (&acc)[8][8], int32_t (&acq)[8][8]) {
+                                         uint32_t end, uint32_t sq, uint32_t half, Wait next_chunk, Addr next_addr,
+                                         DpFrag (&f)[2], int32_t (&acc)[8][8], int32_t (&acq)[8][8]) {
 #pragma unroll 1
   for (uint32_t o = first; o < end; o += 16) {
     opaque(o);
