@@ -18,8 +18,8 @@
 // - Issue slots: an int8 MMA takes 5 and a chunk's unpack about 500 a warp.
 //
 // Measured against the kernel that ran both pipes in every product warp, whole
-// passes: N=256, F=256, T=16384 5017 -> 4222 us (220 -> 261 effective TOPS);
-// N=8192, F=4, T=2048 9439 -> 7974 us; N=1024, F=64, T=4096 4738 -> 3984 us
+// passes: N=256, F=256, T=16384 5019 -> 4220 us (220 -> 262 effective TOPS);
+// N=8192, F=4, T=2048 9440 -> 7964 us; N=1024, F=64, T=4096 4733 -> 3977 us
 // (schedules the same). Now: tensor pipe 79%, dp4a's pipe 63%, issue 62%.
 //
 // Roles (512 threads, one CTA per SM, launched with 128 registers a thread,
