@@ -65,7 +65,11 @@ int device_setup(int dev) {
   std::lock_guard<std::mutex> lk(g_dev_mu);
   if (dev < 0 || dev >= 64) return fail(CORR_EINVAL, "device ordinal %d out of range", dev);
   if (g_dev_ready[dev]) return CORR_OK;
-  cudaError_t e = cudaSuccess;
+  auto allow_smem = [](const void* k, size_t bytes) {
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+    return e == cudaSuccess ? CORR_OK : fail(CORR_ECUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
+  };
+  int rc;
   for (const void* k : {reinterpret_cast<const void*>(xe::corr_tile_kernel<xe::kSingle, false>),
                         reinterpret_cast<const void*>(xe::corr_tile_kernel<xe::kSingle, false, xe::kSplit7>),
                         reinterpret_cast<const void*>(xe::corr_tile_kernel<xe::kSingle, false, xe::kSplit4>),
@@ -73,20 +77,19 @@ int device_setup(int dev) {
                         reinterpret_cast<const void*>(xe::corr_tile_kernel<xe::kGated, false>),
                         reinterpret_cast<const void*>(xe::corr_tile_kernel<xe::kGateArith, false>),
                         reinterpret_cast<const void*>(xe::corr_tile_kernel<xe::kSingle, true>)})
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemBytes));
+    if ((rc = allow_smem(k, kSmemBytes))) return rc;
+  cudaError_t e;
   for (const void* k : {reinterpret_cast<const void*>(xe::corr_dual_kernel<xe::kSingle>),
                         reinterpret_cast<const void*>(xe::corr_dual_kernel<xe::kBatch>),
                         reinterpret_cast<const void*>(xe::corr_dual_kernel<xe::kGated>),
                         reinterpret_cast<const void*>(xe::corr_dual_kernel<xe::kGateArith>)}) {
     // its register re-split draws on the registers it is launched with: fewer would leave it waiting for good
     cudaFuncAttributes at;
-    e = cudaFuncGetAttributes(&at, k);
-    if (e == cudaSuccess && at.numRegs < xe::kRegsLaunch)
+    if ((e = cudaFuncGetAttributes(&at, k)) != cudaSuccess)
+      return fail(CORR_ECUDA, "cudaFuncGetAttributes: %s", cudaGetErrorString(e));
+    if (at.numRegs < xe::kRegsLaunch)
       return fail(CORR_ECUDA, "the correlator was built with %d registers a thread, not %d", at.numRegs, xe::kRegsLaunch);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kDualSmemBytes));
-    if (e != cudaSuccess) return fail(CORR_ECUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
+    if ((rc = allow_smem(k, kDualSmemBytes))) return rc;
   }
   int bps = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, xe::corr_tile_kernel<xe::kSingle, false>, xe::kThreads,
