@@ -848,17 +848,44 @@ __global__ void __launch_bounds__(kThreads, 1) corr_tile_kernel(const __grid_con
   }
 }
 
-// Copy the bands [f0, f0 + F) of a frame [T][F_in][N] whose rows are not
-// 16-byte aligned into an aligned staging buffer [T][F][Np] (Np = N rounded
-// up to 16); padding bytes are 0x88. rows = T * F; a block copies `per` rows
-// (per * Np near 32 KB). HBM-bound: a thread makes 16 bytes from the up to
-// five aligned words that hold them, so a warp moves 512 bytes with whole
-// words; byte by byte, with a 64-bit division each, the copy took longer than
-// the correlation it prepares. A word is read only if it holds a byte of the
-// row, so it lies in the same page as that byte.
+// 16 bytes of a staged row: `live` bytes of the frame, from byte `at` of it on,
+// then padding (0x88). base = the frame's address, `bytes` its length; word(o)
+// and byte(o) load what lies o bytes into it. They come from the up to five
+// aligned words that hold them; where such a word could reach past the frame's
+// ends, byte by byte, since what lies around a frame is the caller's (and may
+// be no memory at all).
+template <typename Word, typename Byte>
+__host__ __device__ __forceinline__ void stage_16(uint64_t base, int64_t at, int live, int64_t bytes, Word word, Byte byte,
+                                                  uint8_t* dst) {
+  const int off = static_cast<int>((base + static_cast<uint64_t>(at)) & 3);
+  const int64_t w = at - off;
+  if (w < 0 || w + 20 > bytes) {
+#pragma unroll 1
+    for (int k = 0; k < 16; ++k) dst[k] = k < live ? byte(at + k) : static_cast<uint8_t>(0x88);
+    return;
+  }
+  uint32_t v[5], o[4];
+#pragma unroll
+  for (int i = 0; i < 5; ++i) v[i] = 4 * i < live + off ? word(w + 4 * i) : 0u;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int b = live - 4 * i;  // live bytes of this word
+    const uint32_t mask = b >= 4 ? 0xFFFFFFFFu : b <= 0 ? 0u : (1u << (8 * b)) - 1u;
+    const uint32_t x = static_cast<uint32_t>((static_cast<uint64_t>(v[i + 1]) << 32 | v[i]) >> (8 * off));
+    o[i] = (x & mask) | (0x88888888u & ~mask);
+  }
+  *reinterpret_cast<uint4*>(dst) = make_uint4(o[0], o[1], o[2], o[3]);
+}
+
+// Copy the bands [f0, f0 + F) of a frame [T][F_in][N] (`bytes` in all) whose
+// rows are not 16-byte aligned into an aligned staging buffer [T][F][Np] (Np =
+// N rounded up to 16). rows = T * F; a block copies `per` rows (per * Np near
+// 32 KB). HBM-bound: a thread makes 16 bytes, so a warp moves 512 bytes with
+// whole words; byte by byte, with a 64-bit division each, the copy took longer
+// than the correlation it prepares.
 constexpr int kRepackThreads = 256;
 
-__global__ void __launch_bounds__(kRepackThreads) repack_rows_kernel(const uint8_t* __restrict__ src,
+__global__ void __launch_bounds__(kRepackThreads) repack_rows_kernel(const uint8_t* __restrict__ src, int64_t bytes,
                                                                      uint8_t* __restrict__ dst, int64_t rows,
                                                                      int32_t per, int32_t N, int32_t Np, int32_t F,
                                                                      int32_t F_in, int32_t f0) {
@@ -875,20 +902,10 @@ __global__ void __launch_bounds__(kRepackThreads) repack_rows_kernel(const uint8
       const uint32_t t = (fr + r) / static_cast<uint32_t>(F);
       row = (t0 + t) * F_in + f0 + (fr + r - t * F);
     }
-    const uintptr_t a = reinterpret_cast<uintptr_t>(src) + static_cast<uintptr_t>(row * N + e0);
-    const uint32_t* w = reinterpret_cast<const uint32_t*>(a & ~static_cast<uintptr_t>(3));
-    const int off = static_cast<int>(a & 3), live = min(16, N - static_cast<int>(e0));  // bytes of the row here
-    uint32_t v[5];
-#pragma unroll
-    for (int i = 0; i < 5; ++i) v[i] = 4 * i < live + off ? __ldg(w + i) : 0u;
-    uint32_t o[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int b = live - 4 * i;  // live bytes of this word
-      const uint32_t mask = b >= 4 ? 0xFFFFFFFFu : b <= 0 ? 0u : (1u << (8 * b)) - 1u;
-      o[i] = (__funnelshift_r(v[i], v[i + 1], 8 * off) & mask) | (0x88888888u & ~mask);
-    }
-    *reinterpret_cast<uint4*>(dst + (r0 + r) * Np + e0) = make_uint4(o[0], o[1], o[2], o[3]);
+    stage_16(
+        reinterpret_cast<uint64_t>(src), row * N + e0, min(16, N - static_cast<int>(e0)), bytes,
+        [src](int64_t o) { return __ldg(reinterpret_cast<const uint32_t*>(src + o)); },
+        [src](int64_t o) { return __ldg(src + o); }, dst + (r0 + r) * Np + e0);
   }
 }
 

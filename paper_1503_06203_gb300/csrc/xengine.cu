@@ -603,8 +603,8 @@ int stage_if_needed(corr_handle* h, const uint8_t* in, int32_t T, cudaStream_t s
   const int32_t per = std::max(1, 32768 / np);
   const int64_t blocks = ceil_div(rows, per);
   if (blocks > INT32_MAX) return fail(CORR_EINVAL, "frame too large to stage");
-  xe::repack_rows_kernel<<<static_cast<int>(blocks), xe::kRepackThreads, 0, st>>>(in, h->stage, rows, per, h->N, np, h->F,
-                                                                                h->F_in, h->f0);
+  xe::repack_rows_kernel<<<static_cast<int>(blocks), xe::kRepackThreads, 0, st>>>(
+      in, static_cast<int64_t>(T) * h->F_in * h->N, h->stage, rows, per, h->N, np, h->F, h->F_in, h->f0);
   XE_CHECK(h, cudaGetLastError());
   ++h->launches;
   *frame = h->stage;
