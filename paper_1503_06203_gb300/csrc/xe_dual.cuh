@@ -306,6 +306,15 @@ __device__ __forceinline__ void dp_merge(int32_t* part, int lane, int col0, int 
 // The first 16 bytes of a chunk's meta.
 __device__ __forceinline__ int4 meta_head(const DualMeta& m) { return *reinterpret_cast<const int4*>(&m); }
 
+// The next chunk's meta once wait() says that it is there; if that wait ran out,
+// the current one's: the buffer may never have been written, and the operand
+// addresses loaded ahead come from it.
+template <typename Wait, typename Read>
+__host__ __device__ __forceinline__ int4 next_meta(bool& ok, const int4& current, Wait wait, Read read) {
+  ok = wait();
+  return ok ? read() : current;
+}
+
 // ---- the kernel -----------------------------------------------------------------
 template <int kMode>
 __global__ void __launch_bounds__(kDualThreads, 1) corr_dual_kernel(const __grid_constant__ CUtensorMap tmap,
@@ -634,8 +643,8 @@ __global__ void __launch_bounds__(kDualThreads, 1) corr_dual_kernel(const __grid
     }
     int4 next_head = head;
     auto next_chunk = [&](void) {  // waits for the next chunk's planes; its meta
-      ok = mbar_wait_bounded(&sm.pfull[nbuf], nphase, kSpinLimit);
-      next_head = meta_head(sm.pmeta[nbuf]);
+      next_head = next_meta(ok, head, [&] { return mbar_wait_bounded(&sm.pfull[nbuf], nphase, kSpinLimit); },
+                            [&] { return meta_head(sm.pmeta[nbuf]); });
     };
     // samples [first, end), whole k-steps; Q's half of them
     const uint32_t first = 32 * (head.x >> 8), end = min(kTC, (head.z + 31) & ~31), half = (end - first) / 2;
