@@ -600,7 +600,7 @@ int stage_if_needed(corr_handle* h, const uint8_t* in, int32_t T, cudaStream_t s
     h->stage_bytes = need;
   }
   const int64_t rows = static_cast<int64_t>(T) * h->F;
-  const int32_t per = std::max(1, 32768 / np);
+  const int32_t per = xe::repack_rows_per_block(rows, np, g_sms[h->device]);
   const int64_t blocks = ceil_div(rows, per);
   if (blocks > INT32_MAX) return fail(CORR_EINVAL, "frame too large to stage");
   xe::repack_rows_kernel<<<static_cast<int>(blocks), xe::kRepackThreads, 0, st>>>(

@@ -42,11 +42,9 @@ int main(int argc, char** argv) {
 """
 
 
-@pytest.fixture(scope="module")
-def harness(tmp_path_factory):
-    d = tmp_path_factory.mktemp("staging")
+def compiled(d, code):
     src, exe = d / "h.cu", d / "h"
-    src.write_text(HARNESS)
+    src.write_text(code)
     subprocess.run([builder._nvcc(), *builder.ARCH, "-std=c++17", "--extended-lambda", "-I", builder.CSRC, "-I",
                     os.path.join(ROOT, "include"), "-o", str(exe), str(src)], check=True)
     return str(exe)
@@ -57,3 +55,27 @@ def harness(tmp_path_factory):
 def test_only_the_frame_is_read(harness, N, F, T):
     r = subprocess.run([harness, str(N), str(F), str(T)], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout
+
+
+BLOCKS = r"""
+#include <stdio.h>
+#include <stdlib.h>
+#include "xe_corr.cuh"
+int main(int, char** argv) { printf("%d\n", xe::repack_rows_per_block(atoll(argv[1]), atoi(argv[2]), 152)); }
+"""
+
+
+@pytest.fixture(scope="module")
+def blocks(tmp_path_factory):
+    return compiled(tmp_path_factory.mktemp("blocks"), BLOCKS)
+
+
+@pytest.mark.parametrize("N,F,T", [(1, 1, 1), (8, 1, 2048), (8, 256, 64), (30, 1, 640), (65, 16, 200), (250, 3, 128),
+                                   (250, 61, 4001), (1000, 64, 64), (40001, 1, 7)])
+def test_rows_are_spread_over_the_gpu(blocks, N, F, T):
+    rows, Np = T * F, -(-N // 16) * 16
+    per = int(subprocess.run([blocks, str(rows), str(Np)], capture_output=True, text=True, check=True).stdout)
+    steps, n = rows * Np // 16, -(-rows // per)  # 16-byte steps of the frame; blocks of 256 threads
+    assert per >= 1 and (per == 1 or per * Np <= 32768)
+    # every SM has four blocks, or no thread has more than one step (and a row's rounding)
+    assert n >= min(4 * 152 // 2, steps // (256 + Np // 16))
