@@ -87,11 +87,22 @@ struct __align__(128) DualSmem {
   uint8_t box[kDualStages][2][kBoxBytes];          // TMA ring: [stage][A|B][time][element], 64-byte swizzle
   uint8_t plane[kDualBufs][2][3][kPlaneBytes];     // [buffer][A|B][slot][element][time]
   int32_t part[2][kTile * kTile];                  // Re and Im of the item under way, swizzled (part_at)
+  DualMeta meta[kDualStages], pmeta[kDualBufs];    // (from part to here: zero at first, clear_smem)
   uint64_t full[kDualStages], bempty[kDualStages]; // box landed / read by the 4 unpack warps
   uint64_t pfull[kDualBufs], pempty[kDualBufs];    // planes written / read by the 12 product warps
   uint64_t mfull, mempty;                          // dp4a parts added; item written and `part` zero again
-  DualMeta meta[kDualStages], pmeta[kDualBufs];
 };
+
+// Thread k of n's share of the zeroes a CTA starts with: no sums, and no chunk
+// in any buffer. The dp4a warps read a buffer's meta, and load operands at the
+// offset it names, also when the wait for it ran out, so it must never be what
+// shared memory happened to hold. (Not reading it then took 0.5% of every
+// frame, thread 0 clearing it 1%: the loops' code changes with either.)
+__host__ __device__ __forceinline__ void clear_smem(DualSmem& sm, int k, int n) {
+  constexpr int kWords = (sizeof(sm.part) + sizeof(sm.meta) + sizeof(sm.pmeta)) / 4;
+  int32_t* const p = sm.part[0];
+  for (; k < kWords; k += n) p[k] = 0;
+}
 
 // Hides a value's origin from the compiler, which would otherwise split the
 // first or last iteration off the loops below and double their code.
@@ -306,15 +317,6 @@ __device__ __forceinline__ void dp_merge(int32_t* part, int lane, int col0, int 
 // The first 16 bytes of a chunk's meta.
 __device__ __forceinline__ int4 meta_head(const DualMeta& m) { return *reinterpret_cast<const int4*>(&m); }
 
-// The next chunk's meta once wait() says that it is there; if that wait ran out,
-// the current one's: the buffer may never have been written, and the operand
-// addresses loaded ahead come from it.
-template <typename Wait, typename Read>
-__host__ __device__ __forceinline__ int4 next_meta(bool& ok, const int4& current, Wait wait, Read read) {
-  ok = wait();
-  return ok ? read() : current;
-}
-
 // ---- the kernel -----------------------------------------------------------------
 template <int kMode>
 __global__ void __launch_bounds__(kDualThreads, 1) corr_dual_kernel(const __grid_constant__ CUtensorMap tmap,
@@ -341,7 +343,7 @@ __global__ void __launch_bounds__(kDualThreads, 1) corr_dual_kernel(const __grid
     mbar_init(&sm.mempty, kDualMmaWarps);
     fence_barrier_init();
   }
-  for (int k = threadIdx.x; k < 2 * kTile * kTile; k += kDualThreads) sm.part[0][k] = 0;
+  clear_smem(sm, threadIdx.x, kDualThreads);
   // The next launch may set its CTAs up as these leave their SMs; a launch that
   // was allowed to do so waits here for everything before it in its stream.
   launch_dependents();
@@ -643,8 +645,8 @@ __global__ void __launch_bounds__(kDualThreads, 1) corr_dual_kernel(const __grid
     }
     int4 next_head = head;
     auto next_chunk = [&](void) {  // waits for the next chunk's planes; its meta
-      next_head = next_meta(ok, head, [&] { return mbar_wait_bounded(&sm.pfull[nbuf], nphase, kSpinLimit); },
-                            [&] { return meta_head(sm.pmeta[nbuf]); });
+      ok = mbar_wait_bounded(&sm.pfull[nbuf], nphase, kSpinLimit);
+      next_head = meta_head(sm.pmeta[nbuf]);
     };
     // samples [first, end), whole k-steps; Q's half of them
     const uint32_t first = 32 * (head.x >> 8), end = min(kTC, (head.z + 31) & ~31), half = (end - first) / 2;
