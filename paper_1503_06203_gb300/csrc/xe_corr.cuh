@@ -20,6 +20,7 @@
 #pragma once
 #include <cuda.h>
 #include <cstdint>
+#include <type_traits>
 
 #include "xe_ptx.cuh"
 
@@ -851,22 +852,28 @@ __global__ void __launch_bounds__(kThreads, 1) corr_tile_kernel(const __grid_con
 // 16 bytes of a staged row: `live` bytes of the frame, from byte `at` of it on,
 // then padding (0x88). base = the frame's address, `bytes` its length; word(o)
 // and byte(o) load what lies o bytes into it. They come from the up to five
-// aligned words that hold them; where such a word could reach past the frame's
-// ends, byte by byte, since what lies around a frame is the caller's (and may
-// be no memory at all).
-template <typename Word, typename Byte>
+// aligned words that hold them, but from none that reaches past the frame's
+// ends, since what lies around a frame is the caller's (and may be no memory at
+// all): what the frame has of such a word comes byte by byte. kEnds = false:
+// there is no such word.
+template <bool kEnds, typename Word, typename Byte>
 __host__ __device__ __forceinline__ void stage_16(uint64_t base, int64_t at, int live, int64_t bytes, Word word, Byte byte,
                                                   uint8_t* dst) {
   const int off = static_cast<int>((base + static_cast<uint64_t>(at)) & 3);
   const int64_t w = at - off;
-  if (w < 0 || w + 20 > bytes) {
-#pragma unroll 1
-    for (int k = 0; k < 16; ++k) dst[k] = k < live ? byte(at + k) : static_cast<uint8_t>(0x88);
-    return;
-  }
+  const int need = live + off, room = bytes - w < 20 ? static_cast<int>(bytes - w) : 20;
   uint32_t v[5], o[4];
 #pragma unroll
-  for (int i = 0; i < 5; ++i) v[i] = 4 * i < live + off ? word(w + 4 * i) : 0u;
+  for (int i = 0; i < 5; ++i)
+    v[i] = 4 * i < need && (!kEnds || (4 * i + 4 <= room && w + 4 * i >= 0)) ? word(w + 4 * i) : 0u;
+  if (kEnds && (w < 0 || need > (room & ~3))) {
+#pragma unroll
+    for (int i = 0; i < 5; ++i)
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+        if (4 * i + b < room && w + 4 * i + b >= 0 && (4 * i + 4 > room || w + 4 * i < 0))
+          v[i] |= static_cast<uint32_t>(byte(w + 4 * i + b)) << (8 * b);
+  }
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int b = live - 4 * i;  // live bytes of this word
@@ -884,6 +891,7 @@ __host__ __device__ __forceinline__ void stage_16(uint64_t base, int64_t at, int
 // byte, with a 64-bit division each, the copy took longer than the correlation
 // it prepares.
 constexpr int kRepackThreads = 256;
+constexpr int64_t kEndRows = 3;
 
 // Rows a block copies: 32 KB where the frame has enough of them, fewer where
 // that would leave SMs without four blocks, but one step for every thread. A
@@ -898,7 +906,7 @@ inline int32_t repack_rows_per_block(int64_t rows, int32_t Np, int sms) {
   return static_cast<int32_t>(per < most ? per : most);
 }
 
-__global__ void __launch_bounds__(kRepackThreads) repack_rows_kernel(const uint8_t* __restrict__ src, int64_t bytes,
+__global__ void __launch_bounds__(kRepackThreads, 8) repack_rows_kernel(const uint8_t* __restrict__ src, int64_t bytes,
                                                                      uint8_t* __restrict__ dst, int64_t rows,
                                                                      int32_t per, int32_t N, int32_t Np, int32_t F,
                                                                      int32_t F_in, int32_t f0) {
@@ -907,18 +915,35 @@ __global__ void __launch_bounds__(kRepackThreads) repack_rows_kernel(const uint8
   const uint32_t quads = static_cast<uint32_t>(Np) >> 4;
   const int64_t t0 = r0 / F;
   const uint32_t fr = static_cast<uint32_t>(r0 - t0 * F);
-#pragma unroll 4
-  for (uint32_t k = threadIdx.x; k < n * quads; k += kRepackThreads) {
-    const uint32_t r = k / quads, e0 = 16 * (k - r * quads);
-    int64_t row = r0 + r;  // row of the source frame
-    if (F != F_in) {
-      const uint32_t t = (fr + r) / static_cast<uint32_t>(F);
-      row = (t0 + t) * F_in + f0 + (fr + r - t * F);
+  auto copy = [&](uint32_t lo, uint32_t hi, auto ends) {  // rows [lo, hi) of the block's
+    constexpr int kUnroll = decltype(ends)::value ? 1 : 4;
+#pragma unroll kUnroll
+    for (uint32_t k = lo * quads + threadIdx.x; k < hi * quads; k += kRepackThreads) {
+      const uint32_t r = k / quads, e0 = 16 * (k - r * quads);
+      int64_t row = r0 + r;  // row of the source frame
+      if (F != F_in) {
+        const uint32_t t = (fr + r) / static_cast<uint32_t>(F);
+        row = (t0 + t) * F_in + f0 + (fr + r - t * F);
+      }
+      stage_16<decltype(ends)::value>(
+          reinterpret_cast<uint64_t>(src), row * N + e0, min(16, N - static_cast<int>(e0)), bytes,
+          [src](int64_t o) { return __ldg(reinterpret_cast<const uint32_t*>(src + o)); },
+          [src](int64_t o) { return __ldg(src + o); }, dst + (r0 + r) * Np + e0);
     }
-    stage_16(
-        reinterpret_cast<uint64_t>(src), row * N + e0, min(16, N - static_cast<int>(e0)), bytes,
-        [src](int64_t o) { return __ldg(reinterpret_cast<const uint32_t*>(src + o)); },
-        [src](int64_t o) { return __ldg(src + o); }, dst + (r0 + r) * Np + e0);
+  };
+  // Words that reach past the frame's ends belong to its first and last kEndRows rows at most. A block with them
+  // copies those rows apart from the others, or all its rows so if that is one step a thread.
+  const int64_t left = rows - kEndRows - r0;  // the block's rows before the last ones
+  if (r0 >= kEndRows && left >= n) {
+    copy(0, n, std::false_type());
+  } else if (n * quads <= kRepackThreads) {
+    copy(0, n, std::true_type());
+  } else {
+    const uint32_t head = r0 < kEndRows ? min(n, static_cast<uint32_t>(kEndRows - r0)) : 0;
+    const uint32_t tail = left < n ? max(head, static_cast<uint32_t>(max(left, int64_t(0)))) : n;
+    copy(0, head, std::true_type());
+    copy(head, tail, std::false_type());
+    copy(tail, n, std::true_type());
   }
 }
 

@@ -7,11 +7,12 @@ import pytest
 from conftest import ROOT
 from paper_1503_06203_gb300 import builder
 
-# One staged frame [T][F_in][N] at `base` bytes past an aligned address, step by step; the frame's bytes are
-# k * 37 + 11, its neighbours are absent: a load outside [0, bytes) ends the run with status 1.
+# One frame [T][F][N] at `base` bytes past an aligned address, staged step by step; the
+# frame's bytes are k * 37 + 11, its neighbours are absent: a load outside [0, bytes) ends the run with status 1.
 HARNESS = r"""
 #include <stdio.h>
 #include <stdlib.h>
+#include <vector>
 #include "xe_corr.cuh"
 static int64_t bytes;
 static uint8_t at(int64_t o) {
@@ -23,20 +24,31 @@ static uint8_t at(int64_t o) {
 }
 int main(int argc, char** argv) {
   const int N = atoi(argv[1]), F = atoi(argv[2]), T = atoi(argv[3]), Np = (N + 15) / 16 * 16;
-  bytes = (int64_t)T * F * N;
-  for (uint64_t base = 0; base < 16; ++base)
-    for (int64_t row = 0; row < (int64_t)T * F; ++row)
+  const int64_t rows = (int64_t)T * F;
+  bytes = rows * N;
+  for (uint64_t base = 0; base < 16; ++base) {
+    std::vector<uint4> buf(rows * Np / 16);
+    uint8_t* got = reinterpret_cast<uint8_t*>(buf.data());
+    for (int64_t row = 0; row < rows; ++row)
       for (int e0 = 0; e0 < Np; e0 += 16) {
-        alignas(16) uint8_t got[16];
-        xe::stage_16(base, row * N + e0, N - e0 < 16 ? N - e0 : 16, bytes,
-                     [](int64_t o) { return at(o) | at(o + 1) << 8 | at(o + 2) << 16 | (uint32_t)at(o + 3) << 24; },
-                     [](int64_t o) { return at(o); }, got);
-        for (int k = 0; k < 16; ++k)
-          if (got[k] != (e0 + k < N ? at(row * N + e0 + k) : 0x88)) {
-            printf("base %d row %lld byte %d: %02x\n", (int)base, (long long)row, e0 + k, got[k]);
-            return 1;
-          }
+        auto word = [base](int64_t o) {
+          if ((base + o) & 3) exit(2);
+          return at(o) | at(o + 1) << 8 | at(o + 2) << 16 | (uint32_t)at(o + 3) << 24;
+        };
+        auto byte = [](int64_t o) { return at(o); };
+        const int live = N - e0 < 16 ? N - e0 : 16;
+        if (row < xe::kEndRows || row >= rows - xe::kEndRows)  // (as the kernel)
+          xe::stage_16<true>(base, row * N + e0, live, bytes, word, byte, got + row * Np + e0);
+        else
+          xe::stage_16<false>(base, row * N + e0, live, bytes, word, byte, got + row * Np + e0);
       }
+    for (int64_t row = 0; row < rows; ++row)
+      for (int e = 0; e < Np; ++e)
+        if (got[row * Np + e] != (e < N ? at(row * N + e) : 0x88)) {
+          printf("base %d row %lld byte %d: %02x\n", (int)base, (long long)row, e, got[row * Np + e]);
+          return 1;
+        }
+  }
   return 0;
 }
 """
@@ -50,8 +62,14 @@ def compiled(d, code):
     return str(exe)
 
 
-@pytest.mark.parametrize("N,F,T", [(1, 1, 1), (2, 1, 1), (3, 1, 2), (4, 1, 1), (15, 1, 1), (16, 1, 1), (17, 1, 1), (18, 2, 3),
-                                   (31, 1, 2), (64, 1, 2), (66, 3, 2)])
+@pytest.fixture(scope="module")
+def harness(tmp_path_factory):
+    return compiled(tmp_path_factory.mktemp("staging"), HARNESS)
+
+
+@pytest.mark.parametrize("N,F,T", [(1, 1, 1), (2, 1, 1), (1, 5, 1), (1, 2, 3), (7, 1, 1), (3, 1, 2), (4, 1, 1), (15, 1, 1), (16, 1, 1), (17, 1, 1), (18, 2, 3),
+                                   (31, 1, 2), (64, 1, 2), (66, 3, 2), (1, 4, 6), (2, 1, 9), (5, 1, 8),
+                                   (19, 3, 4), (64, 1, 9)])
 def test_only_the_frame_is_read(harness, N, F, T):
     r = subprocess.run([harness, str(N), str(F), str(T)], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout
