@@ -133,8 +133,14 @@ constexpr int kLagStreamThreads = 256;
 // second row of a block, a fixed distance after its first, never wraps: its
 // source addresses are the first row's plus an immediate (N=256, F=256, T=8192:
 // 213.5 -> 206.8 us; address sums were 2 of some 4.5 instructions a byte).
+// Frames of one quad (N = 16) that keep every CTA slot busy don't repeat it:
+// three of four lanes are idle and the copies, a whole box for 16 bytes a row,
+// are what bounds them (N=16, F=256, T=8192: 75 us without, 85 with the ninth
+// box; F=1: 12.3 and 11.5).
 constexpr int kLagBoxBytes = kLagRingBytes / kLagRing;
-constexpr int kLagStreamSmem = kLagRingBytes + kLagBoxBytes + 128;  // dynamic shared memory (aligned to 128 inside)
+constexpr int lag_stream_smem(bool twice) {  // dynamic shared memory (aligned to 128 inside)
+  return kLagRingBytes + (twice ? kLagBoxBytes : 0) + 128;
+}
 
 template <int kW>
 struct LagGeom {
@@ -160,25 +166,26 @@ struct LagStreamArgs {
 
 __device__ __forceinline__ int64_t clamp64(int64_t v, int64_t lo, int64_t hi) { return v < lo ? lo : (v > hi ? hi : v); }
 
-// One lane's 16 output bytes of rows t and t + kPassRows (see the bank note
-// above): visiting step w reads word (w + rot) & 3 of the lane's quad;
-// kInterior = every source row of the block lies inside the frame.
-template <int kW, bool kInterior>
-__device__ __forceinline__ void lag_pair(const uint8_t* ring, int32_t t, const uint32_t (&c)[16],
-                                         const int32_t (&lg)[16], int rot, int32_t T, uint4 (&o)[2]) {
+// One lane's 16 output bytes of row t, or (kRows = 2) of rows t and
+// t + kPassRows (see the bank note above): visiting step w reads word
+// (w + rot) & 3 of the lane's quad; kInterior = every source row of the block
+// lies inside the frame.
+template <int kW, int kRows, bool kInterior>
+__device__ __forceinline__ void lag_rows(const uint8_t* ring, int32_t t, const uint32_t (&c)[16],
+                                         const int32_t (&lg)[16], int rot, int32_t T, uint4 (&o)[kRows]) {
   constexpr int kStep = LagGeom<kW>::kPassRows;
   static_assert(kStep * kW <= kLagBoxBytes, "the second row stays within the repeated slot");
   const uint32_t tb = static_cast<uint32_t>(t & (LagGeom<kW>::kRR - 1)) * kW;
-  uint32_t wv[2][4];
+  uint32_t wv[kRows][4];
 #pragma unroll
   for (int w = 0; w < 4; ++w) {
-    uint32_t v[2][4];
+    uint32_t v[kRows][4];
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
       const int k = 4 * w + b;
       const uint8_t* a = ring + ((tb + c[k]) & (kLagRingBytes - 1u));
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
+      for (int h = 0; h < kRows; ++h) {
         v[h][b] = a[h * kStep * kW];
         if (!kInterior) {
           const int64_t src = static_cast<int64_t>(t) + h * kStep - lg[k];
@@ -187,11 +194,11 @@ __device__ __forceinline__ void lag_pair(const uint8_t* ring, int32_t t, const u
       }
     }
 #pragma unroll
-    for (int h = 0; h < 2; ++h) wv[h][w] = v[h][0] | (v[h][1] << 8) | (v[h][2] << 16) | (v[h][3] << 24);
+    for (int h = 0; h < kRows; ++h) wv[h][w] = v[h][0] | (v[h][1] << 8) | (v[h][2] << 16) | (v[h][3] << 24);
   }
   // undo the rotation: output word j was read at step (j - rot) & 3
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
+  for (int h = 0; h < kRows; ++h) {
     o[h].x = rot == 0 ? wv[h][0] : rot == 1 ? wv[h][3] : rot == 2 ? wv[h][2] : wv[h][1];
     o[h].y = rot == 0 ? wv[h][1] : rot == 1 ? wv[h][0] : rot == 2 ? wv[h][3] : wv[h][2];
     o[h].z = rot == 0 ? wv[h][2] : rot == 1 ? wv[h][1] : rot == 2 ? wv[h][0] : wv[h][3];
@@ -199,7 +206,8 @@ __device__ __forceinline__ void lag_pair(const uint8_t* ring, int32_t t, const u
   }
 }
 
-template <int kW>
+// kTwice: ring slot 0 is repeated behind the ring, and a lane's two rows share their address sums.
+template <int kW, bool kTwice>
 __global__ void __launch_bounds__(kLagStreamThreads, 3) shift_lags_stream_kernel(const __grid_constant__ CUtensorMap map,
                                                                               const LagStreamArgs a) {
   using G = LagGeom<kW>;
@@ -279,7 +287,7 @@ __global__ void __launch_bounds__(kLagStreamThreads, 3) shift_lags_stream_kernel
     lim = min(lim, last);
     for (; next <= lim; ++next) {
       uint64_t* bar = &full[next % kLagRing];
-      const bool twice = next % kLagRing == 0;  // slot 0, and its copy behind the ring
+      const bool twice = kTwice && next % kLagRing == 0;  // slot 0, and its copy behind the ring
       mbar_arrive_expect_tx(bar, static_cast<uint32_t>((twice ? 2 : 1) * kLagBoxBytes));
       tma_load_3d(ring + (next % kLagRing) * kLagBoxBytes, &map, bar, i0, f, static_cast<int32_t>(next * G::kBR));
       if (twice) tma_load_3d(ring + kLagRingBytes, &map, bar, i0, f, static_cast<int32_t>(next * G::kBR));
@@ -307,15 +315,20 @@ __global__ void __launch_bounds__(kLagStreamThreads, 3) shift_lags_stream_kernel
     if (tid == 0 && any) issue_upto(lo + kLagRing - 1);
     const bool interior = t0 - lmax >= 0 && t0 + G::kBR - 1 - lmin < a.T;
     const int32_t tt = static_cast<int32_t>(t0) + warp * G::kR + rr;
-    if (quad_live && tt < t_end) {
-      uint4 o[2];
+    constexpr int kRows = kTwice ? 2 : 1;
+#pragma unroll
+    for (int r = 0; r < 2; r += kRows) {
+      const int32_t t = tt + r * G::kPassRows;
+      if (!quad_live || t >= t_end) break;
+      uint4 o[kRows];
       if (interior)
-        lag_pair<kW, true>(ring, tt, c, lg, rot, a.T, o);
+        lag_rows<kW, kRows, true>(ring, t, c, lg, rot, a.T, o);
       else
-        lag_pair<kW, false>(ring, tt, c, lg, rot, a.T, o);
-      uint8_t* dst = out_base + static_cast<int64_t>(tt) * row_stride;
-      *reinterpret_cast<uint4*>(dst) = o[0];
-      if (tt + G::kPassRows < t_end) *reinterpret_cast<uint4*>(dst + G::kPassRows * row_stride) = o[1];
+        lag_rows<kW, kRows, false>(ring, t, c, lg, rot, a.T, o);
+      uint8_t* dst = out_base + static_cast<int64_t>(t) * row_stride;
+#pragma unroll
+      for (int h = 0; h < kRows; ++h)
+        if (h == 0 || t + h * G::kPassRows < t_end) *reinterpret_cast<uint4*>(dst + h * G::kPassRows * row_stride) = o[h];
     }
   }
   if (fault && tid == 0) {

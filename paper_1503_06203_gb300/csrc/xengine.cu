@@ -1590,6 +1590,14 @@ int32_t* g_lag_err_host = nullptr;
 int32_t* g_lag_err_dev = nullptr;
 int g_lag_ctas_per_sm[64] = {};
 
+// The streaming kernel for element blocks of kw, with or without the repeated slot.
+using LagKernel = void (*)(const CUtensorMap, const xe::LagStreamArgs);
+static LagKernel lag_kernel(int kw, bool twice) {
+  return kw == 128 ? xe::shift_lags_stream_kernel<128, true>
+         : twice   ? xe::shift_lags_stream_kernel<64, true>
+                   : xe::shift_lags_stream_kernel<64, false>;
+}
+
 int lag_stream_setup(int dev) {
   std::lock_guard<std::mutex> lk(g_lag_mu);
   if (!g_lag_err_host) {
@@ -1604,12 +1612,13 @@ int lag_stream_setup(int dev) {
   }
   if (!g_lag_ctas_per_sm[dev]) {
     int bps = 1 << 30;
-    for (const void* k : {reinterpret_cast<const void*>(xe::shift_lags_stream_kernel<64>),
-                          reinterpret_cast<const void*>(xe::shift_lags_stream_kernel<128>)}) {
-      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, xe::kLagStreamSmem);
+    for (int v = 0; v < 3; ++v) {
+      const void* k = reinterpret_cast<const void*>(lag_kernel(v == 0 ? 128 : 64, v != 2));
+      const int smem = xe::lag_stream_smem(v != 2);
+      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
       if (e != cudaSuccess) return fail(CORR_ECUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
       int b = 0;
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k, xe::kLagStreamThreads, xe::kLagStreamSmem);
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k, xe::kLagStreamThreads, smem);
       if (e != cudaSuccess || b < 1) return fail(CORR_ECUDA, "occupancy query: %s", cudaGetErrorString(e));
       bps = std::min(bps, b);
     }
@@ -1654,10 +1663,8 @@ int corr_shift_lags(const uint8_t* in_dev, uint8_t* out_dev, int32_t N, int32_t 
     rc = make_tmap(&tm, in_dev, N, F, T, static_cast<uint32_t>(kw), static_cast<uint32_t>(8192 / kw));
     if (rc) return rc;
     xe::LagStreamArgs la{in_dev, out_dev, lags_dev, N, F, T, static_cast<int32_t>(tseg), g_lag_err_dev};
-    if (kw == 128)
-      xe::shift_lags_stream_kernel<128><<<static_cast<unsigned>(ctas), xe::kLagStreamThreads, xe::kLagStreamSmem, st>>>(tm, la);
-    else
-      xe::shift_lags_stream_kernel<64><<<static_cast<unsigned>(ctas), xe::kLagStreamThreads, xe::kLagStreamSmem, st>>>(tm, la);
+    const bool twice = N > 16 || ctas <= slots;  // (see kLagBoxBytes)
+    lag_kernel(kw, twice)<<<static_cast<unsigned>(ctas), xe::kLagStreamThreads, xe::lag_stream_smem(twice), st>>>(tm, la);
   } else {
     const int64_t ctas = ceil_div(N, 64) * F * ceil_div(T, xe::kLagTB);
     if (ctas > INT32_MAX) return fail(CORR_EINVAL, "shift_lags: frame too large");
