@@ -290,11 +290,14 @@ int64_t corr_plan_tiles(int32_t N, int32_t tile, int32_t* bi_out, int32_t* bj_ou
 
 /*
  * corr_plan_schedule -- host-only scheduler query (no CUDA calls): the work
- * items the library launches for a frame of N, F, T on `ctas` resident CTAs.
- * Tiles are 64 x 64, band-major, row-major over each band's upper triangle
- * (Sec. II.C); time is cut into 128-sample chunks, and into `split` equal
- * ranges of chunks when whole tiles would leave the CTAs unbalanced. Item k
- * is {band f, bi | bj << 16, first chunk, end chunk} (4 int32 each in
+ * items the library launches for the frame of N, F, T that an integration
+ * starts with, on `ctas` resident CTAs (frames added onto it may be cut finer,
+ * since nothing is zeroed for them). Tiles are 64 x 64, band-major, row-major
+ * over each band's upper triangle (Sec. II.C); time is cut into 128-sample
+ * chunks. Where whole tiles alone would leave the CTAs unbalanced, as many of
+ * them as fill every CTA evenly come first (the last round's diagonal tiles
+ * before its others) and the other tiles' time axis is cut into ranges. Item
+ * k is {band f, bi | bj << 16, first chunk, end chunk} (4 int32 each in
  * items_out, at most items_cap items); CTA c runs items c, c + grid, ...
  * *grid_out (if non-NULL) receives the grid size. Returns the item count, or
  * CORR_EINVAL.

@@ -152,11 +152,19 @@ void triangle_tiles(int32_t N, int32_t tile, std::vector<int32_t>& bi, std::vect
 
 }  // namespace
 
-// A launch schedule: work items (band, tile, chunk range) taken round-robin
-// by the CTAs of one persistent launch.
-struct Plan {
+// Work items (band, tile, chunk range) taken round-robin by the CTAs of one
+// persistent launch; split: ranges of the cut tiles' time axis (1: none cut).
+struct WorkList {
   int4* d_items = nullptr;  // {f, bi | bj << 16, c0, c1}
-  int32_t nitems = 0, nch = 0, grid = 0, T = 0, split = 1;
+  int32_t nitems = 0, grid = 0, split = 1;
+};
+
+// A frame's launch schedules: of the frame that an integration starts with,
+// and of those added onto it where that is another one.
+struct Plan {
+  WorkList store, add;
+  int32_t nch = 0, T = 0;
+  const WorkList& list(bool fresh) const { return fresh || !add.d_items ? store : add; }
 };
 
 // ---- the handle ----------------------------------------------------------------
@@ -241,27 +249,35 @@ void frame_tiles(int32_t N, int32_t F, std::vector<int2>& tiles, std::vector<dou
   }
 }
 
-// Items of a frame: its first `whole` tiles over all chunks, the other tiles'
-// time axis cut into `ranges` ranges of whole chunks (range-major, each range
-// over those tiles in frame order). With diag_first the last `slots` whole
-// tiles are dealt diagonal ones (the cheaper ones) first, so that the CTAs
-// that take a range after them are those with time left. CTA k of P takes items k, k+P, ... so the
-// CTAs running together work on neighbouring tiles of one band over the same
-// time range and share its input in L2.
 bool diagonal(const int2& t) { return (t.y & 0xFFFF) == (t.y >> 16); }
 
-void make_items(const std::vector<int2>& tiles, int64_t nch, int64_t slots, int64_t whole, int64_t ranges,
-                bool diag_first, std::vector<int4>& items) {
+// How a frame's tiles are scheduled: the first `whole` tiles over all chunks,
+// the other tiles' time axis cut into `ranges` ranges of whole chunks.
+struct Schedule {
+  int64_t whole = 0, ranges = 1;
+  bool diag_first = false;
+  bool operator!=(const Schedule& o) const {
+    return whole != o.whole || ranges != o.ranges || diag_first != o.diag_first;
+  }
+};
+
+// The work items of a schedule: the whole tiles, then range by range the cut
+// ones in frame order. With diag_first the last `slots` whole tiles are dealt
+// diagonal ones (the cheaper ones) first, so that the CTAs that take a range
+// after them are those with time left. CTA k of P takes items k, k+P, ... so
+// the CTAs running together work on neighbouring tiles of one band over the
+// same time range and share its input in L2.
+void make_items(const std::vector<int2>& tiles, int64_t nch, int64_t slots, const Schedule& sc, std::vector<int4>& items) {
   items.clear();
   const int64_t n = static_cast<int64_t>(tiles.size());
-  items.reserve(static_cast<size_t>(whole + (n - whole) * ranges));
-  for (int64_t u = 0; u < whole; ++u) items.push_back(make_int4(tiles[u].x, tiles[u].y, 0, static_cast<int32_t>(nch)));
-  if (whole == n) return;
-  if (diag_first && whole >= slots)
+  items.reserve(static_cast<size_t>(sc.whole + (n - sc.whole) * sc.ranges));
+  for (int64_t u = 0; u < sc.whole; ++u) items.push_back(make_int4(tiles[u].x, tiles[u].y, 0, static_cast<int32_t>(nch)));
+  if (sc.whole == n) return;
+  if (sc.diag_first && sc.whole >= slots)
     std::stable_partition(items.end() - slots, items.end(), [](const int4& w) { return diagonal(make_int2(w.x, w.y)); });
-  const int64_t per = ceil_div(nch, ranges);
+  const int64_t per = ceil_div(nch, sc.ranges);
   for (int64_t c0 = 0; c0 < nch; c0 += per)
-    for (int64_t u = whole; u < n; ++u)
+    for (int64_t u = sc.whole; u < n; ++u)
       items.push_back(make_int4(tiles[u].x, tiles[u].y, static_cast<int32_t>(c0),
                                 static_cast<int32_t>(std::min<int64_t>(nch, c0 + per))));
 }
@@ -269,122 +285,153 @@ void make_items(const std::vector<int2>& tiles, int64_t nch, int64_t slots, int6
 // Time of an item beside its chunks (filling its pipeline, merging the two
 // engines' sums, writing the tile), in chunks of an off-diagonal tile.
 constexpr double kItemCost = 0.8;
-// Zeroing the output that cut tiles add onto (a launch of its own), in chunks.
-constexpr double kCutCost = 1.0;
+// Zeroing the output that cut tiles add onto (before the first frame of an
+// integration only), in chunks: a launch of its own, and the bytes, kZeroBytes
+// in a chunk's 2 us. Without the bytes N=1024, F=17, T=640 cleared 71 MB to
+// spread 32 of 2312 tiles (203 us, whole tiles only 196), and N=2048, F=3,
+// T=512 50 MB (119 and 114.5).
+constexpr double kCutCost = 1.0, kZeroBytes = 20e6;
 
-// Pick the schedule: whole tiles only (no atomics), if that keeps the busiest
+double zero_cost(int32_t N, int32_t F) { return kCutCost + 4.0 * N * (N + 1.0) * F / kZeroBytes; }
+
+// Pick a frame's schedules, the first one for frames stored into a fresh
+// integration, the second for frames added onto it, which cut tiles without
+// zeroing anything. Whole tiles only (no atomics), if that keeps the busiest
 // CTA within 3% of an even share; else the best of: as many whole tiles as
 // fill every CTA a times over (a, a - 1 or 0 times), the remaining tiles' time
 // axis cut into ranges that occupy every CTA, at most 4 items each. An item's
 // own cost counts, so a short frame is not cut into items that do little
 // else: N=256, F=16, T=1024 (160 tiles of 8 chunks on 152 CTAs) was 1280 items
-// of one chunk, and is 152 whole tiles and 64 such items (41.5 -> 37.1 us a frame).
-void plan_items(int32_t N, int32_t F, int32_t T, int64_t slots, std::vector<int4>& items, int64_t* split_out,
-                int64_t* grid_out, int64_t forced_split = 0) {
-  std::vector<int2> tiles;
-  std::vector<double> cost;
-  frame_tiles(N, F, tiles, cost);
+// of one chunk, and is 152 whole tiles and 32 items of two.
+void choose_schedules(int32_t N, int32_t F, int64_t nch, int64_t slots, const std::vector<int2>& tiles,
+                      const std::vector<double>& cost, Schedule (&out)[2]) {
   const int64_t ntiles = static_cast<int64_t>(tiles.size());
-  const int64_t nch = ceil_div(T, xe::kTC);
-  int64_t best_whole = ntiles, best_ranges = 1;
-  bool best_first = false;
-  if (forced_split > 0) {
-    best_ranges = std::min<int64_t>(forced_split, nch);
-    best_whole = best_ranges > 1 ? 0 : ntiles;
-  } else {
-    double total = 0.0;
-    for (double c : cost) total += c * static_cast<double>(nch) + kItemCost;
-    std::vector<double> load(static_cast<size_t>(slots));
-    // the busiest CTA's cost over an even share, items dealt round-robin
-    auto eff_of = [&](int64_t whole, int64_t ranges, bool diag_first) {
-      std::fill(load.begin(), load.end(), 0.0);
-      const int64_t per = ceil_div(nch, ranges), rem = ntiles - whole;
-      const int64_t P = std::min(slots, whole + rem * ceil_div(nch, per));
-      int64_t k = 0;
-      auto deal = [&](double c) {
-        load[k] += c + kItemCost;
-        if (++k == P) k = 0;
-      };
-      for (int64_t u = 0; u < whole - (diag_first ? slots : 0); ++u) deal(cost[u] * static_cast<double>(nch));
-      for (int diag = 1; diag_first && diag >= 0; --diag)  // (as make_items)
-        for (int64_t u = whole - slots; u < whole; ++u)
-          if (diagonal(tiles[u]) == (diag == 1)) deal(cost[u] * static_cast<double>(nch));
-      for (int64_t c0 = 0; rem && c0 < nch; c0 += per)
-        for (int64_t u = whole; u < ntiles; ++u) deal(cost[u] * static_cast<double>(std::min(per, nch - c0)));
-      return (*std::max_element(load.begin(), load.end()) + (rem ? kCutCost : 0.0)) * static_cast<double>(slots) / total;
+  const double extra[2] = {zero_cost(N, F), 0.0};
+  double total = 0.0;
+  for (double c : cost) total += c * static_cast<double>(nch) + kItemCost;
+  std::vector<double> load(static_cast<size_t>(slots));
+  // the busiest CTA's cost, items dealt round-robin
+  auto most_of = [&](const Schedule& sc) {
+    std::fill(load.begin(), load.end(), 0.0);
+    const int64_t per = ceil_div(nch, sc.ranges), rem = ntiles - sc.whole;
+    const int64_t P = std::min(slots, sc.whole + rem * ceil_div(nch, per));
+    int64_t k = 0;
+    auto deal = [&](double c) {
+      load[k] += c + kItemCost;
+      if (++k == P) k = 0;
     };
-    double best = eff_of(ntiles, 1, false);
-    const int64_t full = ntiles / slots;
-    for (int64_t a = full; best > 1.03 && a >= 0 && a >= full - 2; --a) {
-      const int64_t whole = (a == full - 2 ? 0 : a) * slots, rem = ntiles - whole;
-      if (rem == 0) continue;
-      std::vector<int64_t> ranges = {2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64};
-      for (int64_t k = 1; k <= 2; ++k) ranges.push_back(std::min<int64_t>(64, k * slots / rem));
-      for (int64_t r : ranges) {
-        if (r < 2 || r > nch || rem * r > std::max<int64_t>(4 * slots, 2 * rem)) continue;
-        for (int first = 0; first <= (whole ? 1 : 0); ++first) {
-          const double eff = eff_of(whole, r, first);
-          if (eff < best - 1e-9) {
-            best = eff;
-            best_whole = whole;
-            best_ranges = r;
-            best_first = first;
+    for (int64_t u = 0; u < sc.whole - (sc.diag_first ? slots : 0); ++u) deal(cost[u] * static_cast<double>(nch));
+    for (int diag = 1; sc.diag_first && diag >= 0; --diag)  // (as make_items)
+      for (int64_t u = sc.whole - slots; u < sc.whole; ++u)
+        if (diagonal(tiles[u]) == (diag == 1)) deal(cost[u] * static_cast<double>(nch));
+    for (int64_t c0 = 0; rem && c0 < nch; c0 += per)
+      for (int64_t u = sc.whole; u < ntiles; ++u) deal(cost[u] * static_cast<double>(std::min(per, nch - c0)));
+    return *std::max_element(load.begin(), load.end());
+  };
+  out[0] = out[1] = Schedule{ntiles, 1, false};
+  double best[2];
+  best[0] = best[1] = most_of(out[0]);
+  if (best[0] * static_cast<double>(slots) <= 1.03 * total) return;
+  const int64_t full = ntiles / slots;
+  for (int64_t a = full; a >= 0 && a >= full - 2; --a) {
+    Schedule sc;
+    sc.whole = (a == full - 2 ? 0 : a) * slots;
+    const int64_t rem = ntiles - sc.whole;
+    if (rem == 0) continue;
+    std::vector<int64_t> ranges = {2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64};
+    for (int64_t k = 1; k <= 2; ++k) ranges.push_back(std::min<int64_t>(64, k * slots / rem));
+    ranges.push_back(std::min<int64_t>(64, nch));
+    for (int64_t r : ranges) {
+      if (r < 2 || r > nch || rem * r > std::max<int64_t>(4 * slots, 2 * rem)) continue;
+      sc.ranges = r;
+      for (int first = 0; first <= (sc.whole ? 1 : 0); ++first) {
+        sc.diag_first = first;
+        const double most = most_of(sc);
+        for (int k = 0; k < 2; ++k)
+          if (best[k] * static_cast<double>(slots) > 1.03 * total && most + extra[k] < best[k] - 1e-9 * total) {
+            best[k] = most + extra[k];
+            out[k] = sc;
           }
-        }
       }
     }
   }
-  make_items(tiles, nch, slots, best_whole, best_ranges, best_first, items);
-  *split_out = best_whole == ntiles ? 1 : best_ranges;
-  *grid_out = std::min<int64_t>(slots, static_cast<int64_t>(items.size()));
+}
+
+// The schedules of a frame of T samples (see choose_schedules), or both of
+// `forced_split` ranges.
+void plan_frame(int32_t N, int32_t F, int32_t T, int64_t slots, int64_t forced_split, std::vector<int2>& tiles,
+                Schedule (&out)[2]) {
+  std::vector<double> cost;
+  frame_tiles(N, F, tiles, cost);
+  const int64_t nch = ceil_div(T, xe::kTC);
+  if (forced_split > 0) {
+    const int64_t r = std::min<int64_t>(forced_split, nch);
+    out[0] = out[1] = Schedule{r > 1 ? 0 : static_cast<int64_t>(tiles.size()), r, false};
+  } else {
+    choose_schedules(N, F, nch, slots, tiles, cost, out);
+  }
 }
 
 // The same choice by the items' number alone (every tile counted as an
-// off-diagonal one), for a caller that schedules on every call: whole tiles
-// for whole rounds of the CTAs (or none), the others cut into `ranges`.
-void quick_split(int64_t ntiles, int64_t nch, int64_t slots, int64_t max_items, int64_t* whole, int64_t* ranges) {
-  *whole = ntiles;
-  *ranges = 1;
+// off-diagonal one), for a caller that schedules on every call and stores:
+// whole tiles for whole rounds of the CTAs (or none), the others cut.
+Schedule quick_schedule(int32_t N, int32_t F, int64_t ntiles, int64_t nch, int64_t slots, int64_t max_items) {
+  Schedule out{ntiles, 1, false};
   double best = static_cast<double>(ceil_div(ntiles, slots)) * (static_cast<double>(nch) + kItemCost);
   for (int64_t w : {ntiles / slots * slots, int64_t(0)}) {
     const int64_t rem = ntiles - w;
     if (rem == 0) continue;
-    for (int64_t r : {2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64}) {
-      if (r > nch || w + rem * r > max_items) break;
-      const double t = static_cast<double>(w / slots) * (static_cast<double>(nch) + kItemCost) + kCutCost +
+    for (int64_t r : {int64_t(2), int64_t(3), int64_t(4), int64_t(6), int64_t(8), int64_t(12), int64_t(16), int64_t(24),
+                      int64_t(32), int64_t(48), int64_t(64), std::min<int64_t>(64, nch)}) {
+      if (r < 2 || r > nch || w + rem * r > max_items) continue;
+      const double t = static_cast<double>(w / slots) * (static_cast<double>(nch) + kItemCost) + zero_cost(N, F) +
                        static_cast<double>(ceil_div(rem * r, slots)) * (static_cast<double>(ceil_div(nch, r)) + kItemCost);
       if (t < best) {
         best = t;
-        *whole = w;
-        *ranges = r;
+        out = Schedule{w, r, false};
       }
     }
   }
+  return out;
+}
+
+// CTAs resident at a time on a device.
+int64_t slots_of(int dev) { return static_cast<int64_t>(g_sms[dev]) * g_blocks_per_sm[dev]; }
+
+// One of a plan's work lists on the device.
+int upload_items(corr_handle* h, const std::vector<int2>& tiles, int64_t nch, int64_t slots, const Schedule& sc, WorkList* l) {
+  std::vector<int4> items;
+  make_items(tiles, nch, slots, sc, items);
+  if (items.size() > static_cast<size_t>(INT32_MAX)) return fail(CORR_EINVAL, "schedule too large");
+  cudaError_t ae = cudaMalloc(&l->d_items, items.size() * sizeof(int4));
+  if (ae != cudaSuccess) {
+    l->d_items = nullptr;
+    return alloc_failed("work list", items.size() * sizeof(int4), ae);
+  }
+  XE_CHECK(h, cudaMemcpy(l->d_items, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice));
+  l->nitems = static_cast<int32_t>(items.size());
+  l->grid = static_cast<int32_t>(std::min<int64_t>(slots, l->nitems));
+  l->split = static_cast<int32_t>(sc.whole == static_cast<int64_t>(tiles.size()) ? 1 : sc.ranges);
+  return CORR_OK;
 }
 
 // Schedule a frame of T samples for the resident CTAs of this device.
 int build_plan(corr_handle* h, int32_t T, Plan* pl) {
-  const int64_t slots = static_cast<int64_t>(g_sms[h->device]) * g_blocks_per_sm[h->device];
-  std::vector<int4> items;
-  int64_t split = 1, grid = 1;
-  plan_items(h->N, h->F, T, slots, items, &split, &grid, h->split_opt);
-  if (items.size() > static_cast<size_t>(INT32_MAX)) return fail(CORR_EINVAL, "schedule too large");
-  cudaError_t ae = cudaMalloc(&pl->d_items, items.size() * sizeof(int4));
-  if (ae != cudaSuccess) {
-    pl->d_items = nullptr;
-    return alloc_failed("work list", items.size() * sizeof(int4), ae);
-  }
-  XE_CHECK(h, cudaMemcpy(pl->d_items, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice));
-  pl->nitems = static_cast<int32_t>(items.size());
-  pl->nch = static_cast<int32_t>(ceil_div(T, xe::kTC));
-  pl->grid = static_cast<int32_t>(grid);
+  const int64_t slots = slots_of(h->device), nch = ceil_div(T, xe::kTC);
+  std::vector<int2> tiles;
+  Schedule sc[2];
+  plan_frame(h->N, h->F, T, slots, h->split_opt, tiles, sc);
+  int rc = upload_items(h, tiles, nch, slots, sc[0], &pl->store);
+  if (rc) return rc;
+  if (sc[1] != sc[0] && (rc = upload_items(h, tiles, nch, slots, sc[1], &pl->add))) return rc;
+  pl->nch = static_cast<int32_t>(nch);
   pl->T = T;
-  pl->split = static_cast<int32_t>(split);
   return CORR_OK;
 }
 
 void free_plan(Plan* pl) {
-  if (pl->d_items) cudaFree(pl->d_items);
+  if (pl->store.d_items) cudaFree(pl->store.d_items);
+  if (pl->add.d_items) cudaFree(pl->add.d_items);
   *pl = Plan();
 }
 
@@ -459,6 +506,7 @@ int launch_frame(corr_handle* h, const uint8_t* frame, int32_t Np, int64_t row_b
   CUtensorMap tm;
   const bool enc = effective_product(h->product) == 2;
   const int hybrid = chunk_hybrid_flag(h->product, h->mma_steps);
+  const WorkList& wl = pl.list(h->fresh && !enc);
   int rc = make_tmap(&tm, frame, Np, h->F, pl.T, xe::kTile, xe::kTC, row_bytes, !enc && hybrid == xe::kSplitDual);
   if (rc) return rc;
   if (enc) {
@@ -483,12 +531,12 @@ int launch_frame(corr_handle* h, const uint8_t* frame, int32_t Np, int64_t row_b
     XE_CHECK(h, cudaGetLastError());
     h->launches += 2;
     h->fresh = false;  // the correlator adds onto the seeded terms
-  } else if (h->fresh && pl.split > 1) {  // time-split items add atomically onto zeros
+  } else if (h->fresh && wl.split > 1) {  // time-split items add atomically onto zeros
     XE_CHECK(h, cudaMemsetAsync(h->acc, 0, static_cast<size_t>(h->F) * h->B * 2 * sizeof(int32_t), st));
   }
   xe::CorrArgs a;
-  a.items = pl.d_items;
-  a.nitems = pl.nitems;
+  a.items = wl.d_items;
+  a.nitems = wl.nitems;
   a.nch = pl.nch;
   a.T = pl.T;
   a.N = h->N;
@@ -498,15 +546,15 @@ int launch_frame(corr_handle* h, const uint8_t* frame, int32_t Np, int64_t row_b
   a.hybrid = hybrid;
   a.err = h->d_err;
   if (enc)  // (the offset-encoded route splits 96 / 32 or runs tensor cores only)
-    xe::corr_tile_kernel<xe::kSingle, true><<<pl.grid, xe::kThreads, kSmemBytes, st>>>(tm, a);
+    xe::corr_tile_kernel<xe::kSingle, true><<<wl.grid, xe::kThreads, kSmemBytes, st>>>(tm, a);
   else if (a.hybrid == xe::kSplit7)
-    xe::corr_tile_kernel<xe::kSingle, false, xe::kSplit7><<<pl.grid, xe::kThreads, kSmemBytes, st>>>(tm, a);
+    xe::corr_tile_kernel<xe::kSingle, false, xe::kSplit7><<<wl.grid, xe::kThreads, kSmemBytes, st>>>(tm, a);
   else if (a.hybrid == xe::kSplitDual)
-    XE_CHECK(h, launch_dual(pl.grid, st, tm, a));
+    XE_CHECK(h, launch_dual(wl.grid, st, tm, a));
   else if (a.hybrid == xe::kSplit4)
-    xe::corr_tile_kernel<xe::kSingle, false, xe::kSplit4><<<pl.grid, xe::kThreads, kSmemBytes, st>>>(tm, a);
+    xe::corr_tile_kernel<xe::kSingle, false, xe::kSplit4><<<wl.grid, xe::kThreads, kSmemBytes, st>>>(tm, a);
   else
-    xe::corr_tile_kernel<xe::kSingle, false><<<pl.grid, xe::kThreads, kSmemBytes, st>>>(tm, a);
+    xe::corr_tile_kernel<xe::kSingle, false><<<wl.grid, xe::kThreads, kSmemBytes, st>>>(tm, a);
   XE_CHECK(h, cudaGetLastError());
   ++h->launches;
   h->fresh = false;
@@ -925,7 +973,7 @@ static int accumulate_alone(corr_handle_t* h, const uint8_t* packed_dev, int32_t
   if ((rc = stage_if_needed(h, packed_dev, T, st, &frame, &np, &row_bytes))) return rc;
   Plan pl = h->plan;
   if (T != h->T) {
-    const int64_t n = pl.nitems;
+    const int64_t n = pl.store.nitems;
     if (h->piece_cap < n) {
       if (h->d_piece) XE_CHECK(h, cudaFreeAsync(h->d_piece, st));
       h->d_piece = nullptr;
@@ -940,10 +988,11 @@ static int accumulate_alone(corr_handle_t* h, const uint8_t* packed_dev, int32_t
     pl.T = T;
     pl.nch = static_cast<int32_t>(ceil_div(T, xe::kTC));
     const int blocks = static_cast<int>(std::min<int64_t>(ceil_div(n, 256), 4 * g_sms[h->device]));
-    piece_items_kernel<<<blocks, 256, 0, st>>>(h->plan.d_items, h->d_piece, n, pl.nch);
+    piece_items_kernel<<<blocks, 256, 0, st>>>(h->plan.store.d_items, h->d_piece, n, pl.nch);
     XE_CHECK(h, cudaGetLastError());
     ++h->launches;
-    pl.d_items = h->d_piece;
+    pl.store.d_items = h->d_piece;
+    pl.add = WorkList();
   }
   if ((rc = launch_frame(h, frame, np, row_bytes, pl, st))) return rc;
   h->samples += T;
@@ -987,7 +1036,7 @@ int batch_impl(corr_handle_t* const* hs, const uint8_t* const* inputs, const int
     corr_handle* h = hs[k];
     const int32_t Tk = Ts ? Ts[k] : h->T;
     const int64_t nb = ceil_div(h->N, xe::kTile);
-    if (Tk <= h->T && (Tk == h->T || h->plan.split == 1) && nb * (nb + 1) / 2 * h->F >= kAloneWaves * slots) {
+    if (Tk <= h->T && (Tk == h->T || h->plan.store.split == 1) && nb * (nb + 1) / 2 * h->F >= kAloneWaves * slots) {
       int rc = accumulate_alone(h, inputs[k], Tk, st);
       if (rc) return rc;
     } else {
@@ -1700,11 +1749,11 @@ int corr_set_option(corr_handle_t* h, int option, int64_t value) {
     h->split_opt = static_cast<int>(value);
     free_plan(&h->plan);
     if ((rc = build_plan(h, h->T, &h->plan))) return rc;
-    if (h->plan_chunk.d_items) {
+    if (h->plan_chunk.T) {
       free_plan(&h->plan_chunk);
       if ((rc = build_plan(h, h->hchunk_T, &h->plan_chunk))) return rc;
     }
-    if (h->plan_tail.d_items) {
+    if (h->plan_tail.T) {
       free_plan(&h->plan_tail);
       if ((rc = build_plan(h, h->tail_T, &h->plan_tail))) return rc;
     }
@@ -1827,9 +1876,11 @@ int64_t corr_plan_tiles(int32_t N, int32_t tile, int32_t* bi_out, int32_t* bj_ou
 int64_t corr_plan_schedule(int32_t N, int32_t F, int32_t T, int32_t ctas, int32_t* items_out, int64_t items_cap,
                            int32_t* grid_out) {
   if (N < 1 || N > CORR_MAX_N || F < 1 || T < 1 || ctas < 1) return fail(CORR_EINVAL, "bad schedule query");
+  std::vector<int2> tiles;
+  Schedule sc[2];
+  plan_frame(N, F, T, ctas, 0, tiles, sc);
   std::vector<int4> items;
-  int64_t split = 1, grid = 1;
-  plan_items(N, F, T, ctas, items, &split, &grid);
+  make_items(tiles, ceil_div(T, xe::kTC), ctas, sc[0], items);
   if (items_out)
     for (int64_t k = 0; k < static_cast<int64_t>(items.size()) && k < items_cap; ++k) {
       items_out[4 * k] = items[k].x;
@@ -1837,7 +1888,7 @@ int64_t corr_plan_schedule(int32_t N, int32_t F, int32_t T, int32_t ctas, int32_
       items_out[4 * k + 2] = items[k].z;
       items_out[4 * k + 3] = items[k].w;
     }
-  if (grid_out) *grid_out = static_cast<int32_t>(grid);
+  if (grid_out) *grid_out = static_cast<int32_t>(std::min<int64_t>(ctas, static_cast<int64_t>(items.size())));
   return static_cast<int64_t>(items.size());
 }
 
@@ -1933,11 +1984,9 @@ extern "C" int corr_correlate_noalloc(const uint8_t* packed_dev, int32_t N, int3
   if ((rc = noalloc_setup(dev, &scratch))) return rc;
   const int64_t slots = static_cast<int64_t>(g_sms[dev]) * g_blocks_per_sm[dev];
   // whole tiles, or cut ones where those leave CTAs idle, within the array and the frame's chunks
-  int64_t whole, split;
-  quick_split(ntiles, nch, slots, kNoAllocMaxItems, &whole, &split);
-  const int64_t per = ceil_div(nch, split);
-  split = ceil_div(nch, per);  // no empty ranges
-  const int64_t nitems = whole + (ntiles - whole) * split;
+  const Schedule sc = quick_schedule(N, F, ntiles, nch, slots, kNoAllocMaxItems);
+  const int64_t whole = sc.whole, per = ceil_div(nch, sc.ranges);
+  const int64_t nitems = whole + (ntiles - whole) * ceil_div(nch, per);  // (no empty ranges)
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t vis_bytes = static_cast<size_t>(F) * (static_cast<size_t>(N) * (N + 1) / 2) * 2 * sizeof(int32_t);
   // the fault word starts at zero; time-split items add atomically onto a zeroed output
