@@ -530,14 +530,29 @@ int zero_sums(corr_handle* h, int32_t* p, size_t bytes, cudaStream_t st) {
   return CORR_OK;
 }
 
+// Stored tiles of one chunk with 33 to 128 samples, two or more a CTA, run on
+// corr_tile_kernel at share 6: such an item is over before its end is paid for,
+// and there the dual-engine kernel's tensor warps write a tile out of shared
+// memory after the dp4a warps added theirs (2 us), while 16 product warps
+// store from registers. N=256, F=256: T=64 54.7 -> 45.4 us, T=128 66.5 -> 56.4;
+// N=1024, F=64: 174 -> 160, 217 -> 185; N=8192, F=3: 487 -> 461, 605 -> 515.
+// Up to 32 samples (dp4a idle) and where tiles are added to (both kernels the
+// same within a few per cent) the dual-engine kernel stays, and for fewer
+// tiles, where consecutive frames overlap: N=64, F=64, T=128 6.3 against 6.2 us,
+// T=96 5.8 against 8.2.
+bool short_stores(int hybrid, bool fresh, int64_t ntiles, int64_t nch, int32_t T, int64_t slots) {
+  return hybrid == xe::kSplitDual && fresh && nch == 1 && T > 32 && ntiles >= 2 * slots;
+}
+
 // Launch the correlator over the handle's F bands of Np bytes (16-byte
 // aligned rows) at `frame`, time samples row_bytes apart.
 int launch_frame(corr_handle* h, const uint8_t* frame, int32_t Np, int64_t row_bytes, const Plan& pl,
                  cudaStream_t st) {
   CUtensorMap tm;
   const bool enc = effective_product(h->product) == 2;
-  const int hybrid = chunk_hybrid_flag(h->product, h->mma_steps);
+  int hybrid = chunk_hybrid_flag(h->product, h->mma_steps);
   const WorkList& wl = pl.list(h->fresh && !enc);
+  if (!enc && short_stores(hybrid, h->fresh, wl.nitems, pl.nch, pl.T, slots_of(h->device))) hybrid = xe::kSplit6;
   int rc = make_tmap(&tm, frame, Np, h->F, pl.T, xe::kTile, xe::kTC, row_bytes, !enc && hybrid == xe::kSplitDual);
   if (rc) return rc;
   if (enc) {
@@ -1114,7 +1129,10 @@ static int batch_shared(corr_handle_t* const* hs, const uint8_t* const* inputs, 
   for (int k = 0; k < n; ++k) order[k] = k;
   std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) { return per[a] > per[b]; });
 
-  const int hybrid = shared_split(chunk_hybrid_flag(hs[0]->product, hs[0]->mma_steps));
+  int hybrid = shared_split(chunk_hybrid_flag(hs[0]->product, hs[0]->mma_steps));
+  bool stores = true;
+  for (int k = 0; k < n && stores; ++k) stores = short_stores(hybrid, hs[k]->fresh, nitems, nch[k], Ts ? Ts[k] : hs[k]->T, slots);
+  if (stores) hybrid = xe::kSplit6;
 
   std::lock_guard<std::mutex> lk(g_batch_mu);
   if (!g_ring[dev]) g_ring[dev] = new (std::nothrow) BatchRing;
@@ -2031,7 +2049,8 @@ extern "C" int corr_correlate_noalloc(const uint8_t* packed_dev, int32_t N, int3
                                           static_cast<int32_t>(per), whole, nitems);
   if ((e = cudaGetLastError()) != cudaSuccess) return fail(CORR_ECUDA, "noalloc plan: %s", cudaGetErrorString(e));
   CUtensorMap tm;
-  if ((rc = make_tmap(&tm, packed_dev, N, F, T, xe::kTile, xe::kTC, 0, true))) return rc;
+  const bool stores = short_stores(xe::kSplitDual, true, ntiles, nch, T, slots);
+  if ((rc = make_tmap(&tm, packed_dev, N, F, T, xe::kTile, xe::kTC, 0, !stores))) return rc;
   xe::CorrArgs a;
   a.items = scratch + 1;
   a.nitems = static_cast<int32_t>(nitems);
@@ -2041,10 +2060,15 @@ extern "C" int corr_correlate_noalloc(const uint8_t* packed_dev, int32_t N, int3
   a.B = static_cast<int64_t>(N) * (N + 1) / 2;
   a.vis = vis_dev;
   a.fresh = 1;
-  a.hybrid = xe::kSplitDual;
+  a.hybrid = stores ? xe::kSplit6 : xe::kSplitDual;
   a.err = reinterpret_cast<int32_t*>(scratch);
   const int grid = static_cast<int>(std::min<int64_t>(slots, nitems));
-  e = launch_dual(grid, st, tm, a);
+  if (stores) {
+    xe::corr_tile_kernel<xe::kSingle, false><<<grid, xe::kThreads, kSmemBytes, st>>>(tm, a);
+    e = cudaGetLastError();
+  } else {
+    e = launch_dual(grid, st, tm, a);
+  }
   if (e != cudaSuccess) return fail(CORR_ECUDA, "noalloc correlate: %s", cudaGetErrorString(e));
   if (status_dev && (e = cudaMemcpyAsync(status_dev, scratch, sizeof(int32_t), cudaMemcpyDeviceToDevice, st)) !=
                         cudaSuccess)
