@@ -875,7 +875,11 @@ __host__ __device__ __forceinline__ void stage_16(uint64_t base, int64_t at, int
   for (int i = 0; i < 4; ++i) {
     const int b = live - 4 * i;  // live bytes of this word
     const uint32_t mask = b >= 4 ? 0xFFFFFFFFu : b <= 0 ? 0u : (1u << (8 * b)) - 1u;
+#ifdef __CUDA_ARCH__
+    const uint32_t x = __funnelshift_r(v[i], v[i + 1], 8 * off);
+#else
     const uint32_t x = static_cast<uint32_t>((static_cast<uint64_t>(v[i + 1]) << 32 | v[i]) >> (8 * off));
+#endif
     o[i] = (x & mask) | (0x88888888u & ~mask);
   }
   *reinterpret_cast<uint4*>(dst) = make_uint4(o[0], o[1], o[2], o[3]);
