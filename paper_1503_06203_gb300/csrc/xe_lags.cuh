@@ -133,10 +133,10 @@ constexpr int kLagStreamThreads = 256;
 // second row of a block, a fixed distance after its first, never wraps: its
 // source addresses are the first row's plus an immediate (N=256, F=256, T=8192:
 // 213.5 -> 206.8 us; address sums were 2 of some 4.5 instructions a byte).
-// Frames of one quad (N = 16) that keep every CTA slot busy don't repeat it:
-// three of four lanes are idle and the copies, a whole box for 16 bytes a row,
-// are what bounds them (N=16, F=256, T=8192: 75 us without, 85 with the ninth
-// box; F=1: 12.3 and 11.5).
+// Frames of one quad (N = 16) with a CTA for every SM don't repeat it: three of
+// four lanes are idle and the copies, a whole box for 16 bytes a row, are what
+// bounds them (N=16, F=256: T=8192 75 us without, 85 with the ninth box, T=256
+// 8.3 and 10.2; F=1, T=2048 12.3 and 11.5).
 constexpr int kLagBoxBytes = kLagRingBytes / kLagRing;
 constexpr int lag_stream_smem(bool twice) {  // dynamic shared memory (aligned to 128 inside)
   return kLagRingBytes + (twice ? kLagBoxBytes : 0) + 128;

@@ -1761,7 +1761,7 @@ int corr_shift_lags(const uint8_t* in_dev, uint8_t* out_dev, int32_t N, int32_t 
     rc = make_tmap(&tm, in_dev, N, F, T, static_cast<uint32_t>(kw), static_cast<uint32_t>(8192 / kw));
     if (rc) return rc;
     xe::LagStreamArgs la{in_dev, out_dev, lags_dev, N, F, T, static_cast<int32_t>(tseg), g_lag_err_dev};
-    const bool twice = N > 16 || ctas <= slots;  // (see kLagBoxBytes)
+    const bool twice = N > 16 || ctas <= g_sms[dev];  // (see kLagBoxBytes)
     lag_kernel(kw, twice)<<<static_cast<unsigned>(ctas), xe::kLagStreamThreads, xe::lag_stream_smem(twice), st>>>(tm, la);
   } else {
     const int64_t ctas = ceil_div(N, 64) * F * ceil_div(T, xe::kLagTB);
