@@ -160,7 +160,8 @@ struct WorkList {
 };
 
 // A frame's launch schedules: of the frame that an integration starts with,
-// and of those added onto it where that is another one.
+// and of those added onto it where that is another one. One allocation, at
+// store.d_items, holds both.
 struct Plan {
   WorkList store, add;
   int32_t nch = 0, T = 0;
@@ -398,32 +399,31 @@ Schedule quick_schedule(int32_t N, int32_t F, int64_t ntiles, int64_t nch, int64
 // CTAs resident at a time on a device.
 int64_t slots_of(int dev) { return static_cast<int64_t>(g_sms[dev]) * g_blocks_per_sm[dev]; }
 
-// One of a plan's work lists on the device.
-int upload_items(corr_handle* h, const std::vector<int2>& tiles, int64_t nch, int64_t slots, const Schedule& sc, WorkList* l) {
-  std::vector<int4> items;
-  make_items(tiles, nch, slots, sc, items);
-  if (items.size() > static_cast<size_t>(INT32_MAX)) return fail(CORR_EINVAL, "schedule too large");
-  cudaError_t ae = cudaMalloc(&l->d_items, items.size() * sizeof(int4));
-  if (ae != cudaSuccess) {
-    l->d_items = nullptr;
-    return alloc_failed("work list", items.size() * sizeof(int4), ae);
-  }
-  XE_CHECK(h, cudaMemcpy(l->d_items, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice));
-  l->nitems = static_cast<int32_t>(items.size());
-  l->grid = static_cast<int32_t>(std::min<int64_t>(slots, l->nitems));
-  l->split = static_cast<int32_t>(sc.whole == static_cast<int64_t>(tiles.size()) ? 1 : sc.ranges);
-  return CORR_OK;
-}
-
 // Schedule a frame of T samples for the resident CTAs of this device.
 int build_plan(corr_handle* h, int32_t T, Plan* pl) {
   const int64_t slots = slots_of(h->device), nch = ceil_div(T, xe::kTC);
   std::vector<int2> tiles;
   Schedule sc[2];
   plan_frame(h->N, h->F, T, slots, h->split_opt, tiles, sc);
-  int rc = upload_items(h, tiles, nch, slots, sc[0], &pl->store);
-  if (rc) return rc;
-  if (sc[1] != sc[0] && (rc = upload_items(h, tiles, nch, slots, sc[1], &pl->add))) return rc;
+  std::vector<int4> items[2];
+  WorkList* list[2] = {&pl->store, &pl->add};
+  for (int k = 0; k < (sc[1] != sc[0] ? 2 : 1); ++k) {
+    make_items(tiles, nch, slots, sc[k], items[k]);
+    if (items[k].size() > static_cast<size_t>(INT32_MAX)) return fail(CORR_EINVAL, "schedule too large");
+    list[k]->nitems = static_cast<int32_t>(items[k].size());
+    list[k]->grid = static_cast<int32_t>(std::min<int64_t>(slots, list[k]->nitems));
+    list[k]->split = static_cast<int32_t>(sc[k].whole == static_cast<int64_t>(tiles.size()) ? 1 : sc[k].ranges);
+  }
+  const size_t stored = items[0].size();
+  items[0].insert(items[0].end(), items[1].begin(), items[1].end());
+  const size_t bytes = items[0].size() * sizeof(int4);
+  cudaError_t ae = cudaMalloc(&pl->store.d_items, bytes);
+  if (ae != cudaSuccess) {
+    pl->store.d_items = nullptr;
+    return alloc_failed("work list", bytes, ae);
+  }
+  if (!items[1].empty()) pl->add.d_items = pl->store.d_items + stored;
+  XE_CHECK(h, cudaMemcpy(pl->store.d_items, items[0].data(), bytes, cudaMemcpyHostToDevice));
   pl->nch = static_cast<int32_t>(nch);
   pl->T = T;
   return CORR_OK;
@@ -431,7 +431,6 @@ int build_plan(corr_handle* h, int32_t T, Plan* pl) {
 
 void free_plan(Plan* pl) {
   if (pl->store.d_items) cudaFree(pl->store.d_items);
-  if (pl->add.d_items) cudaFree(pl->add.d_items);
   *pl = Plan();
 }
 
