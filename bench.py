@@ -138,17 +138,24 @@ def kernel_source_hash() -> str:
     return h.hexdigest()[:16]
 
 
-def effective_split(N: int, F: int, T: int, split: int, ctas: int) -> int:
-    """The time split a launch actually uses (0 = the library's automatic choice for this shape)."""
+def effective_split(N: int, F: int, T: int, split: int, ctas: int) -> str:
+    """The time split of the frame that an integration starts with (0 = the library's automatic choice for this
+    shape): the ranges every tile is cut into ("1": none is cut), or "W+CxR" for W whole tiles and C cut into R."""
+    nch = -(-T // 128)
     if split > 0:
-        return min(split, -(-T // 128))
+        return str(min(split, nch))
     import paper_1503_06203_gb300 as xe
     items, _ = xe.plan_schedule(N, F, T, ctas)
     nb = -(-N // 64)
-    return len(items) // (nb * (nb + 1) // 2 * F)
+    tiles = nb * (nb + 1) // 2 * F
+    whole = int(((items[:, 2] == 0) & (items[:, 3] == nch)).sum())
+    if whole == tiles:
+        return "1"
+    ranges = (len(items) - whole) // (tiles - whole)
+    return f"{whole}+{tiles - whole}x{ranges}" if whole else str(ranges)
 
 
-def recorded_traffic(workload: str, product: int, split: int, mma_steps: int):
+def recorded_traffic(workload: str, product: int, split: str, mma_steps: int):
     """DRAM bytes per launch from the committed ncu summary of this workload, if taken on the current
     kernel source with the same launch knobs (a time split changes the writers' traffic; `split` is the
     effective split, see effective_split)."""
