@@ -1875,37 +1875,44 @@ int corr_dims(const corr_handle_t* h, int32_t* N, int32_t* F, int32_t* T) {
 
 const char* corr_last_error(void) { return g_last_error.c_str(); }
 
+// Destroying reports nothing, so a call that fails there (an event last recorded
+// in a captured graph cannot be waited for) leaves no error behind either: the
+// next launch's check would take it for its own.
+static void quiet(cudaError_t e) {
+  if (e != cudaSuccess) cudaGetLastError();
+}
+
 void corr_destroy(corr_handle_t* h) {
   if (!h) return;
-  if (h->has_last) cudaEventSynchronize(h->last);
+  if (h->has_last) quiet(cudaEventSynchronize(h->last));
   for (int k = 0; k < 2; ++k)
     if (h->ev_copied_out[k]) {
-      cudaEventSynchronize(h->ev_copied_out[k]);  // overlapped readouts still copying out
-      cudaEventDestroy(h->ev_copied_out[k]);
+      quiet(cudaEventSynchronize(h->ev_copied_out[k]));  // overlapped readouts still copying out
+      quiet(cudaEventDestroy(h->ev_copied_out[k]));
     }
   if (h->acc_alt) {  // both sets: free the library's, leave a caller-owned one to the caller
-    cudaFree(h->acc_alt);
+    quiet(cudaFree(h->acc_alt));
     h->acc = h->acc_own;
   }
-  if (h->own_acc && h->acc) cudaFree(h->acc);
-  if (h->d_err) cudaFree(h->d_err);
+  if (h->own_acc && h->acc) quiet(cudaFree(h->acc));
+  if (h->d_err) quiet(cudaFree(h->d_err));
   free_plan(&h->plan);
   free_plan(&h->plan_chunk);
   free_plan(&h->plan_tail);
-  if (h->stage) cudaFree(h->stage);
-  if (h->d_sums) cudaFree(h->d_sums);
-  if (h->d_piece) cudaFree(h->d_piece);
+  if (h->stage) quiet(cudaFree(h->stage));
+  if (h->d_sums) quiet(cudaFree(h->d_sums));
+  if (h->d_piece) quiet(cudaFree(h->d_piece));
   for (int k = 0; k < 2; ++k) {
-    if (h->hchunk[k]) cudaFree(h->hchunk[k]);
-    if (h->ev_copied[k]) cudaEventDestroy(h->ev_copied[k]);
-    if (h->ev_used[k]) cudaEventDestroy(h->ev_used[k]);
+    if (h->hchunk[k]) quiet(cudaFree(h->hchunk[k]));
+    if (h->ev_copied[k]) quiet(cudaEventDestroy(h->ev_copied[k]));
+    if (h->ev_used[k]) quiet(cudaEventDestroy(h->ev_used[k]));
   }
-  if (h->ev_in) cudaEventDestroy(h->ev_in);
-  if (h->s_status) cudaStreamDestroy(h->s_status);
-  if (h->h_status) cudaFreeHost(h->h_status);
-  if (h->s_copy) cudaStreamDestroy(h->s_copy);
-  if (h->s_comp) cudaStreamDestroy(h->s_comp);
-  if (h->last) cudaEventDestroy(h->last);
+  if (h->ev_in) quiet(cudaEventDestroy(h->ev_in));
+  if (h->s_status) quiet(cudaStreamDestroy(h->s_status));
+  if (h->h_status) quiet(cudaFreeHost(h->h_status));
+  if (h->s_copy) quiet(cudaStreamDestroy(h->s_copy));
+  if (h->s_comp) quiet(cudaStreamDestroy(h->s_comp));
+  if (h->last) quiet(cudaEventDestroy(h->last));
   delete h;
 }
 
