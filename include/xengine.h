@@ -229,7 +229,9 @@ int corr_shift_lags(const uint8_t* in_dev, uint8_t* out_dev, int32_t N, int32_t 
  *     tiles with bi == bj). Single-frame calls (corr_accumulate,
  *     corr_accumulate_host) on product path 1 take every share; batched and
  *     gated calls take 8, 6 or 5 and product path 2 takes 8 or 6 (other values
- *     run as 6).
+ *     run as 6). Frames of 33 to 128 samples that start an integration run 5
+ *     as 6 where they have two or more tiles a CTA (so does
+ *     corr_correlate_noalloc).
  * A batched launch takes its product path and share from its first handle.
  * Returns CORR_OK, CORR_EINVAL or CORR_EBUSY.
  */

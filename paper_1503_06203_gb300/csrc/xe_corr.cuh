@@ -1,5 +1,6 @@
-// The correlator kernel of product paths 0 and 2 and of the shares other than
-// the default (which xe_dual.cuh runs), and what both kernels share: TMA-staged
+// The correlator kernel of product paths 0 and 2, of the shares other than the
+// default (which xe_dual.cuh runs) and of the default's short stored frames
+// (short_stores in xengine.cu), and what both kernels share: TMA-staged
 // 4-bit input, excess-8 unpack into K-major int8 planes in shared memory,
 // integer Hermitian product in the three-product form, packed upper-triangle
 // writer.

@@ -252,7 +252,8 @@ __device__ __forceinline__ void dp_load(uint32_t ra, uint32_t rb, DpFrag& n) {
 // current ones. On a diagonal tile only the 36 of 64 row/column block pairs
 // with entries i <= j are computed. Off the diagonal the column side's two
 // words sit swapped (unpack), so that a dp4a's two operands come from
-// different register banks (5% on the loop).
+// different register banks (without it N=8192, F=1, T=2048 takes 2001 us
+// instead of 1925, N=256, F=256, T=16384 4317 instead of 4203).
 template <bool kDiag>
 __device__ __forceinline__ void dp_step(uint32_t ra, uint32_t rb, DpFrag& n, const DpFrag& f, int32_t (&acc)[8][8]) {
 #pragma unroll

@@ -434,11 +434,11 @@ void free_plan(Plan* pl) {
   *pl = Plan();
 }
 
-// swizzled: 16-byte pieces of a 64-byte box row are exchanged by a pattern of the
-// row (the dual-engine kernel's boxes).
 // 3-D map (elements, bands, time) of F bands of Np bytes starting at `base`;
 // consecutive time samples are row_bytes apart (0: F * Np, a frame of exactly
 // these bands). Elements past Np and samples past T read as zero bytes.
+// swizzled: 16-byte pieces of a 64-byte box row are exchanged by a pattern of
+// the row (the dual-engine kernel's boxes).
 int make_tmap(CUtensorMap* m, const uint8_t* base, int32_t Np, int32_t F, int32_t T, uint32_t box_n = xe::kTile,
               uint32_t box_t = xe::kTC, int64_t row_bytes = 0, bool swizzled = false) {
   EncodeTiledFn enc = encode_fn();
