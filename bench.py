@@ -51,8 +51,8 @@ WORKLOADS = {
 EXTRA_WORKLOADS = ("batched", "batched_small", "served", "lags_gates")
 KERNEL_SOURCES = ["paper_1503_06203_gb300/csrc/xe_dual.cuh", "paper_1503_06203_gb300/csrc/xe_corr.cuh",
                   "paper_1503_06203_gb300/csrc/xe_ptx.cuh"]
-TRAFFIC_FILES = {"pathfinder": os.path.join(ROOT, "profiles", "corr_tile_kernel_pathfinder.md"),
-                 "large_n": os.path.join(ROOT, "profiles", "corr_tile_kernel_large_n.md")}
+TRAFFIC_FILES = {"pathfinder": os.path.join(ROOT, "profiles", "corr_dual_kernel_pathfinder.md"),
+                 "large_n": os.path.join(ROOT, "profiles", "corr_dual_kernel_large_n.md")}
 MEASURED_PEAKS = os.path.join(ROOT, "MEASURED_PEAKS.json")
 SERVED_RATES = "10,40,80"
 

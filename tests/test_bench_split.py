@@ -21,3 +21,12 @@ def bench():
 ])
 def test_effective_split(bench, N, F, T, split, name):
     assert bench.effective_split(N, F, T, split, 152) == name
+
+
+@pytest.mark.parametrize("workload,shape", [("pathfinder", (256, 256, 16384)), ("large_n", (8192, 4, 2048))])
+def test_traffic_record_is_of_this_kernel(bench, workload, shape):
+    split = bench.effective_split(*shape, 0, 152)
+    N, F, T = shape
+    moved = N * F * T + 4 * N * (N + 1) * F
+    assert 0.9 * moved < bench.recorded_traffic(workload, 1, split, 5) < 1.1 * moved
+    assert bench.recorded_traffic(workload, 1, "152+8x4", 5) is None and bench.recorded_traffic(workload, 1, split, 6) is None
