@@ -535,10 +535,11 @@ int zero_sums(corr_handle* h, int32_t* p, size_t bytes, cudaStream_t st) {
 // memory after the dp4a warps added theirs (2 us), while 16 product warps
 // store from registers. N=256, F=256: T=64 54.7 -> 45.4 us, T=128 66.5 -> 56.4;
 // N=1024, F=64: 174 -> 160, 217 -> 185; N=8192, F=3: 487 -> 461, 605 -> 515.
-// Up to 32 samples (dp4a idle) and where tiles are added to (both kernels the
-// same within a few per cent) the dual-engine kernel stays, and for fewer
-// tiles, where consecutive frames overlap: N=64, F=64, T=128 6.3 against 6.2 us,
-// T=96 5.8 against 8.2.
+// Up to 32 samples (dp4a idle: N=8192, F=3, T=24 437 against 504 us) and where
+// tiles are added to (each is faster on some sizes: N=8192, F=3, T=128 697
+// against 761, N=256, F=256, T=128 71 against 65) the dual-engine kernel stays,
+// and for fewer tiles, where consecutive frames overlap: N=64, F=64, T=96 5.8
+// against 8.2 us.
 bool short_stores(int hybrid, bool fresh, int64_t ntiles, int64_t nch, int32_t T, int64_t slots) {
   return hybrid == xe::kSplitDual && fresh && nch == 1 && T > 32 && ntiles >= 2 * slots;
 }
