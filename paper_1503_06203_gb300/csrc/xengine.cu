@@ -332,9 +332,11 @@ void choose_schedules(int32_t N, int32_t F, int64_t nch, int64_t slots, const st
   out[0] = out[1] = Schedule{ntiles, 1, false};
   double best[2];
   best[0] = best[1] = most_of(out[0]);
-  if (best[0] * static_cast<double>(slots) <= 1.03 * total) return;
   const int64_t full = ntiles / slots;
   for (int64_t a = full; a >= 0 && a >= full - 2; --a) {
+    bool open[2];  // not within 3% yet
+    for (int k = 0; k < 2; ++k) open[k] = best[k] * static_cast<double>(slots) > 1.03 * total;
+    if (!open[0] && !open[1]) return;
     Schedule sc;
     sc.whole = (a == full - 2 ? 0 : a) * slots;
     const int64_t rem = ntiles - sc.whole;
@@ -349,7 +351,7 @@ void choose_schedules(int32_t N, int32_t F, int64_t nch, int64_t slots, const st
         sc.diag_first = first;
         const double most = most_of(sc);
         for (int k = 0; k < 2; ++k)
-          if (best[k] * static_cast<double>(slots) > 1.03 * total && most + extra[k] < best[k] - 1e-9 * total) {
+          if (open[k] && most + extra[k] < best[k] - 1e-9 * total / static_cast<double>(slots)) {
             best[k] = most + extra[k];
             out[k] = sc;
           }
@@ -399,14 +401,16 @@ Schedule quick_schedule(int32_t N, int32_t F, int64_t ntiles, int64_t nch, int64
 // CTAs resident at a time on a device.
 int64_t slots_of(int dev) { return static_cast<int64_t>(g_sms[dev]) * g_blocks_per_sm[dev]; }
 
-// Schedule a frame of T samples for the resident CTAs of this device.
+// Schedule a frame of T samples for the resident CTAs of this device. *pl is
+// empty, and stays so on failure.
 int build_plan(corr_handle* h, int32_t T, Plan* pl) {
   const int64_t slots = slots_of(h->device), nch = ceil_div(T, xe::kTC);
   std::vector<int2> tiles;
   Schedule sc[2];
   plan_frame(h->N, h->F, T, slots, h->split_opt, tiles, sc);
   std::vector<int4> items[2];
-  WorkList* list[2] = {&pl->store, &pl->add};
+  Plan np;
+  WorkList* list[2] = {&np.store, &np.add};
   for (int k = 0; k < (sc[1] != sc[0] ? 2 : 1); ++k) {
     make_items(tiles, nch, slots, sc[k], items[k]);
     if (items[k].size() > static_cast<size_t>(INT32_MAX)) return fail(CORR_EINVAL, "schedule too large");
@@ -417,15 +421,17 @@ int build_plan(corr_handle* h, int32_t T, Plan* pl) {
   const size_t stored = items[0].size();
   items[0].insert(items[0].end(), items[1].begin(), items[1].end());
   const size_t bytes = items[0].size() * sizeof(int4);
-  cudaError_t ae = cudaMalloc(&pl->store.d_items, bytes);
-  if (ae != cudaSuccess) {
-    pl->store.d_items = nullptr;
-    return alloc_failed("work list", bytes, ae);
+  cudaError_t e = cudaMalloc(&np.store.d_items, bytes);
+  if (e != cudaSuccess) return alloc_failed("work list", bytes, e);
+  if (!items[1].empty()) np.add.d_items = np.store.d_items + stored;
+  e = cudaMemcpy(np.store.d_items, items[0].data(), bytes, cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) {
+    cudaFree(np.store.d_items);
+    return cuda_fail(h, e, "copying the work list");
   }
-  if (!items[1].empty()) pl->add.d_items = pl->store.d_items + stored;
-  XE_CHECK(h, cudaMemcpy(pl->store.d_items, items[0].data(), bytes, cudaMemcpyHostToDevice));
-  pl->nch = static_cast<int32_t>(nch);
-  pl->T = T;
+  np.nch = static_cast<int32_t>(nch);
+  np.T = T;
+  *pl = np;
   return CORR_OK;
 }
 
