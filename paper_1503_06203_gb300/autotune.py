@@ -40,7 +40,7 @@ def gpu_key() -> str:
     return f"{p.name}|sm_{p.major}{p.minor}|{p.multi_processor_count}sm"
 
 
-TUNER_VERSION = 3  # the candidate set and the kernels it chose among: entries of another version are not reused
+TUNER_VERSION = 4  # the candidate set and the kernels it chose among: entries of another version are not reused
 
 
 def shape_key(N: int, F: int, T: int) -> str:
